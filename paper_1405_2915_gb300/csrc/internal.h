@@ -229,6 +229,8 @@ struct StencilLaunch {
 int launch_stencil(const StencilLaunch &st, const Choice &c, cudaStream_t s);
 // `steps` applications of a 2D forward stencil fused tile-wise, c.tile steps
 // per pass (ping-pong between st.out and tmp, the last pass writes st.out).
+int launch_stream2d(bool taps5, int k, const float *in, float *out, int64_t rows, int64_t cols, int b, const float *w9,
+                    cudaStream_t s);   // k steps in one pass (k_stream.cu)
 int launch_stencil_chain_fused(const StencilLaunch &st, int steps, float *tmp, const Choice &c, cudaStream_t s);
 int chain_variant_count();
 const char *chain_variant_name(int v);
