@@ -82,6 +82,7 @@ __global__ void __launch_bounds__(1024)
 batched_prep(const int64_t *__restrict__ off, int64_t B, int64_t total, int tile, Layout L,
              float *__restrict__ results, Control *ctl, int64_t max_t)
 {
+    dev::grid_wait();
     constexpr int IPT = 4;
     __shared__ int64_t smem[33];
     __shared__ int bad;
@@ -197,6 +198,7 @@ batched_big(const float *__restrict__ values, const int64_t *__restrict__ off, f
             float *__restrict__ scan_out, Layout L, uint64_t *words, int64_t max_t, int64_t total_elems, Control *ctl,
             uint32_t epoch, uint64_t limit_ns)
 {
+    dev::grid_wait();
     extern __shared__ __align__(1024) unsigned char dyn[];   // kBigTile floats
     float *buf = reinterpret_cast<float *>(dyn);
     __shared__ __align__(8) uint64_t bars[kBigSub];   // one per 16 KiB chunk (= sub-tile)
@@ -403,6 +405,7 @@ batched_main(const float *__restrict__ values, const int64_t *__restrict__ off, 
              float *__restrict__ scan_out, Layout L, uint64_t *words, int64_t max_t, Control *ctl, uint32_t epoch,
              uint64_t limit_ns)
 {
+    dev::grid_wait();
     constexpr int TILE = kBlock * 4 * V;
     __shared__ float smem[kBlock / 32 + 1];
     __shared__ float red_smem[32];
@@ -594,6 +597,7 @@ template <int TILE>
 __global__ void __launch_bounds__(kBlock)
 batched_meta(const int64_t *__restrict__ off, Layout L, TileMeta *__restrict__ meta)
 {
+    dev::grid_wait();
     const int64_t total = *reinterpret_cast<volatile int64_t *>(L.total_tiles);
     for (int64_t t = (int64_t)blockIdx.x * kBlock + threadIdx.x; t < total; t += (int64_t)gridDim.x * kBlock) {
         const TileInfo x = tile_info<TILE>(t, total, L, off);
@@ -613,6 +617,7 @@ __global__ void __launch_bounds__(kBlock)
 batched_rts_sums(const float *__restrict__ values, const TileMeta *__restrict__ meta, Layout L, double *aggS,
                  double *aggQ)
 {
+    dev::grid_wait();
     __shared__ float red[32];
     const int64_t total = *reinterpret_cast<volatile int64_t *>(L.total_tiles);
     TileMeta x = blockIdx.x < total ? load_meta(meta, blockIdx.x) : TileMeta{0, 0, 0, 0};
@@ -647,6 +652,7 @@ __global__ void __launch_bounds__(kBlock)
 batched_rts_prefix(Layout L, int64_t B, const double *__restrict__ aggS, const double *__restrict__ aggQ,
                    double *__restrict__ prefS, float *__restrict__ results, int scan, int red)
 {
+    dev::grid_wait();
     const int lane = threadIdx.x & 31;
     const int64_t warps = (int64_t)gridDim.x * (kBlock / 32);
     const int64_t total = *reinterpret_cast<volatile int64_t *>(L.total_tiles);
@@ -676,6 +682,7 @@ __global__ void __launch_bounds__(kBlock, V <= 4 ? 1 : 3)
 batched_rts_apply(const float *__restrict__ values, const TileMeta *__restrict__ meta, float *__restrict__ scan_out,
                   Layout L, const double *__restrict__ prefS)
 {
+    dev::grid_wait();
     __shared__ float smem[kBlock / 32 + 1];
     __shared__ float s_pre[2];
     const int64_t total = *reinterpret_cast<volatile int64_t *>(L.total_tiles);

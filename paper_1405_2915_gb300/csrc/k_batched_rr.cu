@@ -94,6 +94,7 @@ __device__ __forceinline__ int64_t br_instance_of(const int64_t *__restrict__ of
 __global__ void __launch_bounds__(256)
 batched_br_meta(const int64_t *__restrict__ off, int64_t B, int64_t total, BrMeta *__restrict__ meta)
 {
+    dev::grid_wait();
     const int64_t ntiles = (total + kBrTE - 1) / kBrTE;
     for (int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; t < ntiles; t += (int64_t)gridDim.x * blockDim.x) {
         const int64_t last = (t + 1) * kBrTE < total ? (t + 1) * kBrTE - 1 : total - 1;
@@ -107,6 +108,7 @@ __global__ void __launch_bounds__(1024)
 batched_br_prep(const int64_t *__restrict__ off, int64_t B, int64_t total, float *__restrict__ results,
                 int *__restrict__ ok, Control *ctl)
 {
+    dev::grid_wait();
     __shared__ int bad;
     if (threadIdx.x == 0) bad = (off[0] != 0 || off[B] != total) ? 1 : 0;
     __syncthreads();
@@ -129,6 +131,7 @@ batched_br(const float *__restrict__ values, const int64_t *__restrict__ off, in
            const BrMeta *__restrict__ meta, dev::LookbackDesc d, Control *ctl, uint32_t epoch, int64_t skip_tile,
            uint64_t limit_ns)
 {
+    dev::grid_wait();
     constexpr int TE = kBrTE, NA = kBrAggW, QC = kBrQueue, CAP = kBrOffCap;
     constexpr uint32_t TB = TE * 4;
     extern __shared__ __align__(1024) unsigned char dyn[];   // R ring slots, then one buffer per scanner warp

@@ -46,6 +46,7 @@ __global__ void __launch_bounds__(1024)
 batched_seg_prep(const int64_t *__restrict__ off, int64_t B, int64_t total, int tile, float *__restrict__ results,
                  int *__restrict__ ok, int64_t *__restrict__ tile_inst, Control *ctl)
 {
+    dev::grid_wait();
     __shared__ int bad;
     if (threadIdx.x == 0) bad = (off[0] != 0 || off[B] != total) ? 1 : 0;
     __syncthreads();
@@ -74,6 +75,7 @@ batched_seg(const float *__restrict__ values, const int64_t *__restrict__ off, i
             const int64_t *__restrict__ tile_inst, uint64_t *words, int64_t ntiles, Control *ctl, uint32_t epoch,
             uint64_t limit_ns)
 {
+    dev::grid_wait();
     constexpr int NW = kBlock / 32, NS = SUBS + SUBR, TILE = NS * kSubTile, SLEN = SUBS * kSubTile;
     constexpr int PER = (NS * NW + 31) / 32;   // warp ranges per lane in the tile's combine
     extern __shared__ __align__(1024) unsigned char dyn[];   // SUBS x 16 KiB

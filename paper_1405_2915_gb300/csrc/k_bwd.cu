@@ -53,6 +53,7 @@ __device__ __forceinline__ void one(const BwdArgs &p, int64_t i, float gsc)
 template <int FN, bool VEC>
 __global__ void __launch_bounds__(256) map_bwd_kernel(BwdArgs p)
 {
+    dev::grid_wait();
     const float gsc = p.gs_dev ? __ldg(p.gs_dev) : p.gs_host;
     const int64_t stride = (int64_t)gridDim.x * blockDim.x;
     const int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;

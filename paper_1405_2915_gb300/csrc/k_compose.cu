@@ -30,6 +30,7 @@ __global__ void __launch_bounds__(128, 5)
 compose_colwalk(const float *__restrict__ in, int64_t rows, int64_t cols, int b, W9 w, float a,
                 float *__restrict__ partials)
 {
+    dev::grid_wait();
     __shared__ float wsum[4];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int64_t strip0 = ((int64_t)blockIdx.x * 4 + warp) * 128;

@@ -59,6 +59,7 @@ __global__ void __launch_bounds__(256)
 coulomb_direct(const float4 *__restrict__ atoms, int64_t m, float *__restrict__ out, int64_t rows, int64_t cols,
                float h, float z0)
 {
+    dev::grid_wait();
     const int64_t total = rows * cols;
     for (int64_t p = (int64_t)blockIdx.x * 256 + threadIdx.x; p < total; p += (int64_t)gridDim.x * 256) {
         const int64_t i = p / cols, j = p - i * cols;
@@ -89,6 +90,7 @@ __global__ void __launch_bounds__(256)
 coulomb_tiled(const float4 *__restrict__ atoms, int64_t m, float *__restrict__ out, int64_t rows, int64_t cols,
               float h, float z0)
 {
+    dev::grid_wait();
     __shared__ float4 sa[kChunk];
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
     const int64_t i = (int64_t)blockIdx.y * 8 + w;

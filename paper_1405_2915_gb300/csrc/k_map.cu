@@ -34,6 +34,7 @@ template <int FN>
 __global__ void map_scalar(const float *__restrict__ x, const float *__restrict__ y,
                            float *__restrict__ out, int64_t n, float a)
 {
+    dev::grid_wait();
     const int64_t stride = (int64_t)gridDim.x * blockDim.x;
     for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += stride) {
         float yv = MapF<FN>::nin == 2 ? y[i] : 0.f;
@@ -57,6 +58,7 @@ template <int FN, int EPT, bool HINT>
 __global__ void map_vec(const float *__restrict__ x, const float *__restrict__ y,
                         float *__restrict__ out, int head, int64_t nvec, int tail, float a)
 {
+    dev::grid_wait();
     const int64_t gtid = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     map_edges<FN>(x, y, out, head, nvec, tail, a, gtid);
     const float4 *x4 = reinterpret_cast<const float4 *>(x + head);
@@ -88,6 +90,7 @@ template <int FN, int EPT>
 __global__ void map_vec_grid(const float *__restrict__ x, const float *__restrict__ y,
                              float *__restrict__ out, int head, int64_t nvec, int tail, float a)
 {
+    dev::grid_wait();
     const int64_t gtid = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     map_edges<FN>(x, y, out, head, nvec, tail, a, gtid);
     const float4 *x4 = reinterpret_cast<const float4 *>(x + head);
@@ -123,6 +126,7 @@ __global__ void map_vec_grid(const float *__restrict__ x, const float *__restric
 template <int FN>
 __global__ void map_scalar_inplace(const float *x, const float *y, float *out, int64_t n, float a)
 {
+    dev::grid_wait();
     const int64_t stride = (int64_t)gridDim.x * blockDim.x;
     for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += stride) {
         float yv = MapF<FN>::nin == 2 ? y[i] : 0.f;
@@ -134,6 +138,7 @@ template <int FN, int EPT>
 __global__ void map_vec_inplace(const float *x, const float *y, float *out, int head, int64_t nvec, int tail,
                                 float a)
 {
+    dev::grid_wait();
     const int64_t gtid = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     map_edges<FN>(x, y, out, head, nvec, tail, a, gtid);
     const float4 *x4 = reinterpret_cast<const float4 *>(x + head);

@@ -24,6 +24,7 @@ __device__ __forceinline__ int64_t clampi(int64_t k, int64_t m) { return k < 0 ?
 __global__ void gather_scalar(const float *__restrict__ A, int64_t m, const int32_t *__restrict__ idx,
                               float *__restrict__ out, int64_t n)
 {
+    dev::grid_wait();
     for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x)
         out[i] = __ldg(A + clampi(idx[i], m));
 }
@@ -31,6 +32,7 @@ __global__ void gather_scalar(const float *__restrict__ A, int64_t m, const int3
 __global__ void gather_vec4(const float *__restrict__ A, int64_t m, const int32_t *__restrict__ idx,
                             float *__restrict__ out, int64_t n)
 {
+    dev::grid_wait();
     const int64_t nv = n / 4;
     for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < nv; i += (int64_t)gridDim.x * blockDim.x) {
         const uint4 k = dev::ld_stream(reinterpret_cast<const uint4 *>(idx) + i);
@@ -53,6 +55,7 @@ template <int G>
 __global__ void gather_vec4_multi(const float *__restrict__ A, int64_t m, const int32_t *__restrict__ idx,
                                   float *__restrict__ out, int64_t n)
 {
+    dev::grid_wait();
     const int64_t nv = n / 4;
     const int64_t T = (int64_t)gridDim.x * blockDim.x;
     const uint4 *idx4 = reinterpret_cast<const uint4 *>(idx);
@@ -82,6 +85,7 @@ __global__ void gather_vec4_multi(const float *__restrict__ A, int64_t m, const 
 __global__ void rowdot_thread(const float *__restrict__ A, int64_t m, const float *__restrict__ M,
                               float *__restrict__ out, int64_t n)
 {
+    dev::grid_wait();
     for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
         const float *row = M + i * m;
         float acc = 0.f;
@@ -95,6 +99,7 @@ template <bool VEC>
 __global__ void __launch_bounds__(256)
 rowdot_warp(const float *__restrict__ A, int64_t m, const float *__restrict__ M, float *__restrict__ out, int64_t n)
 {
+    dev::grid_wait();
     const int lane = threadIdx.x & 31;
     const int64_t warps = (int64_t)gridDim.x * 8;
     for (int64_t i = (int64_t)blockIdx.x * 8 + (threadIdx.x >> 5); i < n; i += warps) {
@@ -136,6 +141,7 @@ template <bool VEC>
 __global__ void __launch_bounds__(256)
 rowdot_block(const float *__restrict__ A, int64_t m, const float *__restrict__ M, float *__restrict__ out, int64_t n)
 {
+    dev::grid_wait();
     __shared__ float smem[32];
     for (int64_t i = blockIdx.x; i < n; i += gridDim.x) {
         const float *row = M + i * m;
@@ -165,6 +171,7 @@ __global__ void __launch_bounds__(256)
 rowdot_split(const float *__restrict__ A, int64_t m, const float *__restrict__ M, float *__restrict__ part,
              int64_t chunk)
 {
+    dev::grid_wait();
     __shared__ float smem[32];
     const int64_t i = blockIdx.y, S = gridDim.x;
     const int64_t c0 = (int64_t)blockIdx.x * chunk;
@@ -203,6 +210,7 @@ rowdot_split(const float *__restrict__ A, int64_t m, const float *__restrict__ M
 __global__ void __launch_bounds__(256)
 rowdot_combine(const float *__restrict__ part, int64_t S, float *__restrict__ out, int64_t n)
 {
+    dev::grid_wait();
     const int lane = threadIdx.x & 31;
     const int64_t i = (int64_t)blockIdx.x * 8 + (threadIdx.x >> 5);
     if (i >= n) return;

@@ -14,7 +14,7 @@
 namespace skel {
 namespace {
 
-__global__ void probe_empty() {}
+__global__ void probe_empty() { dev::grid_wait(); }
 
 __device__ __forceinline__ uint64_t mix64(uint64_t z)
 {
@@ -29,6 +29,7 @@ __device__ __forceinline__ uint64_t mix64(uint64_t z)
 __global__ void __launch_bounds__(256) probe_l2_random(const float *__restrict__ A, uint32_t mask, int per_thread,
                                                        uint64_t seed, float *__restrict__ sink)
 {
+    dev::grid_wait();
     const uint64_t tid = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x;
     // per-thread stream: a 64-bit linear congruential step (Knuth's MMIX
     // constants) from a hashed start; the index is the state's high bits

@@ -105,6 +105,7 @@ __global__ void __launch_bounds__(BLOCK)
 reduce_phase1(const T *__restrict__ x, const T *__restrict__ y, int64_t n, Span sp,
               T *__restrict__ partials, T *__restrict__ out, Control *ctl, int single_pass)
 {
+    dev::grid_wait();
     __shared__ T smem[32];
     __shared__ int am_last;
     const int64_t nthreads = (int64_t)gridDim.x * BLOCK;
@@ -140,6 +141,7 @@ template <class Op, int BLOCK, class T>
 __global__ void __launch_bounds__(BLOCK)
 reduce_phase2(const T *__restrict__ partials, int count, T *__restrict__ out)
 {
+    dev::grid_wait();
     __shared__ T smem[32];
     T w = Op::id();
     for (int i = threadIdx.x; i < count; i += BLOCK) w = Op::op(w, partials[i]);
@@ -212,7 +214,7 @@ int run_reduce(const ReduceLaunch &r, const Choice &c, cudaStream_t s)
 
 // Writes the identity (n = 0).
 template <class T>
-__global__ void write_scalar(T *out, T v) { *out = v; }
+__global__ void write_scalar(T *out, T v) { dev::grid_wait(); *out = v; }
 
 }  // namespace
 

@@ -92,6 +92,7 @@ scan_lookback(const T *__restrict__ in, T *__restrict__ out, SegGeom g,
               LookbackDesc d, Control *ctl, uint32_t epoch,
               int64_t skip_tile, uint64_t limit_ns)
 {
+    dev::grid_wait();
     using CT = typename ScanTypes<T>::CT;
     constexpr int TILE = kBlock * 4 * V;
     __shared__ T smem[kBlock / 32 + 1];
@@ -200,6 +201,7 @@ __global__ void __launch_bounds__(kBlock)
 scan_tma(const T *__restrict__ in, T *__restrict__ out, SegGeom g, LookbackDesc d, Control *ctl, uint32_t epoch,
          int64_t skip_tile, uint64_t limit_ns)
 {
+    dev::grid_wait();
     using CT = typename ScanTypes<T>::CT;
     using V4 = typename ScanTypes<T>::V4;
     using AddOp = typename std::conditional<std::is_same<T, float>::value, dev::AddF, dev::AddU>::type;
@@ -329,6 +331,7 @@ __global__ void __launch_bounds__(kBlock, SUB == 4 ? 3 : 4)
 scan_big(const T *__restrict__ in, T *__restrict__ out, SegGeom g, LookbackDesc d, Control *ctl, uint32_t epoch,
          int64_t skip_tile, uint64_t limit_ns)
 {
+    dev::grid_wait();
     using CT = typename ScanTypes<T>::CT;
     using V4 = typename ScanTypes<T>::V4;
     extern __shared__ __align__(1024) unsigned char dyn[];   // (SUB * kTmaTile) elements
@@ -553,6 +556,7 @@ __global__ void __launch_bounds__(kBlock, MINB)
 scan_hybrid(const T *__restrict__ in, T *__restrict__ out, SegGeom g, int64_t tpsf, LookbackDesc d, Control *ctl,
             uint32_t epoch, int64_t skip_tile, uint64_t limit_ns)
 {
+    dev::grid_wait();
     using CT = typename ScanTypes<T>::CT;
     using V4 = typename ScanTypes<T>::V4;
     using AddOp = typename std::conditional<std::is_same<T, float>::value, dev::AddF, dev::AddU>::type;
@@ -948,6 +952,7 @@ __global__ void __launch_bounds__(kWsThreads, 1)
 scan_ws(const T *__restrict__ in, T *__restrict__ out, SegGeom g, LookbackDesc d, Control *ctl, uint32_t epoch,
         int64_t skip_tile, uint64_t limit_ns)
 {
+    dev::grid_wait();
     using CT = typename ScanTypes<T>::CT;
     using V4 = typename ScanTypes<T>::V4;
     using AddOp = typename std::conditional<std::is_same<T, float>::value, dev::AddF, dev::AddU>::type;
@@ -1261,6 +1266,7 @@ template <class T, int V>
 __global__ void __launch_bounds__(kBlock)
 scan_tile_sums(const T *__restrict__ in, SegGeom g, typename ScanTypes<T>::CT *__restrict__ sums)
 {
+    dev::grid_wait();
     constexpr int TILE = kBlock * 4 * V;
     __shared__ T smem[kBlock / 32 + 1];
     int64_t first;
@@ -1277,6 +1283,7 @@ template <class CT>
 __global__ void __launch_bounds__(1024)
 scan_tile_prefixes(CT *__restrict__ sums, int64_t tps)
 {
+    dev::grid_wait();
     constexpr int IPT = 8;
     __shared__ CT smem[33];
     CT *s = sums + (int64_t)blockIdx.x * tps;
@@ -1319,6 +1326,7 @@ __global__ void __launch_bounds__(kBlock)
 scan_tile_apply(const T *__restrict__ in, T *__restrict__ out, SegGeom g,
                 const typename ScanTypes<T>::CT *__restrict__ prefixes)
 {
+    dev::grid_wait();
     constexpr int TILE = kBlock * 4 * V;
     __shared__ T smem[kBlock / 32 + 1];
     int64_t first;
@@ -1335,6 +1343,7 @@ template <class T, bool INCL, int V>
 __global__ void __launch_bounds__(kBlock)
 scan_one_block(const T *__restrict__ in, T *__restrict__ out, SegGeom g)
 {
+    dev::grid_wait();
     using CT = typename ScanTypes<T>::CT;
     constexpr int TILE = kBlock * 4 * V;
     __shared__ T smem[kBlock / 32 + 1];

@@ -37,6 +37,7 @@ __global__ void __launch_bounds__(kBlock)
 scan_noalloc_kernel(const T *__restrict__ in, T *__restrict__ out, int64_t n, int64_t ntiles, unsigned char *scratch,
                     int64_t skip_tile, uint64_t limit_ns, bool vec_ok)
 {
+    dev::grid_wait();
     using CT = typename ScanTypes<T>::CT;
     __shared__ T smem[kBlock / 32 + 1];
     __shared__ int64_t s_tile;

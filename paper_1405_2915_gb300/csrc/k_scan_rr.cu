@@ -108,6 +108,7 @@ __global__ void __launch_bounds__((kRrAggW + NC) * 32, 1)
 scan_rr(const T *__restrict__ in, T *__restrict__ out, int64_t seglen, int64_t tps, int64_t ntiles, LookbackDesc d,
         Control *ctl, uint32_t epoch, int64_t skip_tile, uint64_t limit_ns)
 {
+    dev::grid_wait();
     using CT = typename ScanTypes<T>::CT;
     using V4 = typename ScanTypes<T>::V4;
     using AddOp = typename std::conditional<std::is_same<T, float>::value, dev::AddF, dev::AddU>::type;

@@ -84,6 +84,7 @@ template <bool TAPS5>
 __global__ void __launch_bounds__(256)
 st2_smem(const float *__restrict__ in, float *__restrict__ out, int64_t rows, int64_t cols, int b, W9 w)
 {
+    dev::grid_wait();
     __shared__ __align__(16) float s[kSH * kSW];
     const int64_t tx0 = (int64_t)blockIdx.x * kTX, ty0 = (int64_t)blockIdx.y * kTY;
     // stage: kSH rows x kSW/4 groups of 4 columns (cols % 4 == 0: a group is
@@ -119,6 +120,7 @@ __global__ void __launch_bounds__(256)
 st2_tma(const __grid_constant__ CUtensorMap tmap, const float *__restrict__ in, float *__restrict__ out,
         int64_t rows, int64_t cols, int b, W9 w, Control *ctl)
 {
+    dev::grid_wait();
     // dynamic shared memory only (no static shared variables), so the tile
     // starts at the 1024-byte aligned base; the mbarrier follows the tile
     extern __shared__ __align__(1024) unsigned char dyn[];
@@ -169,6 +171,7 @@ template <bool TAPS5, int RH>
 __global__ void __launch_bounds__(128)
 st2_colwalk(const float *__restrict__ in, float *__restrict__ out, int64_t rows, int64_t cols, int b, W9 w)
 {
+    dev::grid_wait();
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int64_t strip0 = ((int64_t)blockIdx.x * 4 + warp) * 128;
     if (strip0 >= cols) return;                     // warp-uniform
@@ -230,6 +233,7 @@ st2_colwalk(const float *__restrict__ in, float *__restrict__ out, int64_t rows,
 template <bool TAPS5>
 __global__ void st2_fold_border(const float *__restrict__ g, float *__restrict__ gin, int64_t rows, int64_t cols, W9 w)
 {
+    dev::grid_wait();
     const int64_t nb = rows == 1 ? cols : (cols == 1 ? rows : 2 * cols + 2 * (rows - 2));
     for (int64_t k = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; k < nb; k += (int64_t)gridDim.x * blockDim.x) {
         int64_t p, q;
@@ -263,6 +267,7 @@ template <int R>
 __global__ void __launch_bounds__(256)
 st1_direct(const float *__restrict__ in, float *__restrict__ out, int64_t n, int b, W33 w)
 {
+    dev::grid_wait();
     for (int64_t i = (int64_t)blockIdx.x * 256 + threadIdx.x; i < n; i += (int64_t)gridDim.x * 256) {
         float acc = 0.f;
 #pragma unroll
@@ -280,6 +285,7 @@ template <int R>
 __global__ void __launch_bounds__(256)
 st1_smem(const float *__restrict__ in, float *__restrict__ out, int64_t n, int b, W33 w)
 {
+    dev::grid_wait();
     constexpr int WV = (k1Per + 2 * R + 3) / 4;        // 16-byte reads per window
     constexpr int SW = k1Tile + 4 * WV;                // window of the last thread stays in bounds
     __shared__ __align__(16) float s[SW];
@@ -335,6 +341,7 @@ template <int R>
 __global__ void __launch_bounds__(256)
 st1_bulk(const float *__restrict__ in, float *__restrict__ out, int64_t n, int b, W33 w, Control *ctl)
 {
+    dev::grid_wait();
     constexpr int HP = (R + 3) / 4 * 4;
     constexpr int NV = 1 + 2 * HP / 4;                 // 16-byte reads per group window
     __shared__ __align__(128) float s[kBT + 2 * HP];
@@ -400,6 +407,7 @@ st1_bulk(const float *__restrict__ in, float *__restrict__ out, int64_t n, int b
 // gin[n-1]): sums w[k] g[i] over outputs i and taps k with clamp(i+k) == p.
 __global__ void st1_fold_ends(const float *__restrict__ g, float *__restrict__ gin, int64_t n, int r, W33 w)
 {
+    dev::grid_wait();
     const int which = threadIdx.x;   // 0: p = 0, 1: p = n-1
     if (which > 1 || (which == 1 && n == 1)) return;
     const int64_t p = which == 0 ? 0 : n - 1;

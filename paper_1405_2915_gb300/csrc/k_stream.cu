@@ -82,6 +82,7 @@ __global__ void __launch_bounds__(32 * kStreamWarps)
 st2_stream(const float *__restrict__ in, float *__restrict__ out, int64_t rows, int64_t cols, int b, W9 w, int H,
            int64_t strips, int64_t nwork)
 {
+    dev::grid_wait();
     using G = StreamGeom<K>;
     constexpr int C = 4, SW = kStreamCols, RING = kStreamRing;
     constexpr uint32_t RB = SW * 4;                     // bytes of a ring row
