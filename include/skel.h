@@ -338,6 +338,25 @@ int skel_compose_map_stencil_sumsq(skel_fn map_fn, const double *params, int npa
                                    const float *weights, int nweights, skel_boundary boundary, skel_handle in,
                                    void *result_host, skel_handle result_dev, void *stream);
 
+/* The composed loss of a grid and its gradient, one pass each (Sec. II, as
+ * above: one implementation for the whole composition):
+ *   t = tanh(x), u = S t, s = the inclusive scan of each row of t,
+ *   loss = sum u^2 + (1/N) sum s^2          (N = rows * cols)
+ *   gx = (S^T (2 g u) + rscan(2 (g/N) s)) * (1 - t^2)
+ * S: the STENCIL9 of skel_mapoverlap (radius 1, weights NULL or 9 values),
+ * S^T its adjoint, rscan the reverse scan of each row.  x, t, gx: 2D F32 of
+ * one shape; loss, g: 1 F32 element; g: the gradient of loss.  The forward
+ * call writes t (NULL: not wanted), which the backward call reads in place of
+ * x.  Equal to the Map, MapOverlap, Scan and MapReduce calls of the
+ * definition within their rounding (the sums are taken in another order).
+ * SKEL_ERR_UNSUPPORTED, with nothing done: PERIODIC, an empty grid, or more
+ * than 8192 columns (a row is held by one thread block); the caller then
+ * makes the separate calls.  Enqueued on `stream`. */
+int skel_composed_loss(const float *weights, int nweights, skel_boundary boundary, skel_handle x, skel_handle t,
+                       skel_handle loss, void *stream);
+int skel_composed_loss_bwd(const float *weights, int nweights, skel_boundary boundary, skel_handle t, skel_handle g,
+                           skel_handle gx, void *stream);
+
 /* MapArray: out[i] = f(A, B[i]) with A read whole (random access) and B per
  * element.  The paper does not define MapArray; the reading used is:
  *   GATHER: A 1D F32 of length m >= 1, B 1D I32 of length n,

@@ -298,6 +298,18 @@ def skel_compose_map_stencil_sumsq(map_fn, stencil, x: Container, params=(), wei
     return res[0] if host else None
 
 
+def skel_composed_loss(weights, boundary, x: Container, t: Container | None, loss: Container, stream=None) -> None:
+    w = _weights(weights)
+    check(lib.skel_composed_loss(w[0], w[1], BOUNDARY[boundary] if isinstance(boundary, str) else boundary, x.handle,
+                                 None if t is None else t.handle, loss.handle, _stream(stream)))
+
+
+def skel_composed_loss_bwd(weights, boundary, t: Container, g: Container, gx: Container, stream=None) -> None:
+    w = _weights(weights)
+    check(lib.skel_composed_loss_bwd(w[0], w[1], BOUNDARY[boundary] if isinstance(boundary, str) else boundary, t.handle,
+                                     g.handle, gx.handle, _stream(stream)))
+
+
 def skel_maparray(fn, whole: Container, elem: Container, out: Container, stream=None) -> None:
     check(lib.skel_maparray(_fn(fn), whole.handle, elem.handle, out.handle, _stream(stream)))
 

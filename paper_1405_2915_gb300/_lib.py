@@ -56,6 +56,8 @@ SIGNATURES = {
     "skel_mapoverlap_chain": (i32, [i32, f32p, i32, i32, i32, vp, vp, vp, vp]),
     "skel_maparray_grid": (i32, [i32, vp, vp, C.POINTER(dbl), i32, vp]),
     "skel_compose_map_stencil_sumsq": (i32, [i32, C.POINTER(dbl), i32, i32, f32p, i32, i32, vp, vp, vp, vp]),
+    "skel_composed_loss": (i32, [f32p, i32, i32, vp, vp, vp, vp]),
+    "skel_composed_loss_bwd": (i32, [f32p, i32, i32, vp, vp, vp, vp]),
     "skel_batched": (i32, [i32, i32, i32, i32, vp, vp, vp, vp, vp]),
     "skel_batched_plan_create": (i32, [i32, i32, i32, i32, vp, vp, vp, vp, vp, C.POINTER(vp)]),
     "skel_plan_launch": (i32, [vp, vp]),

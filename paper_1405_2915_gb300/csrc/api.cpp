@@ -846,6 +846,45 @@ int stencil_common(skel_fn fn, int radius, const float *weights, int nweights, s
                              in->ndim == 1 ? st1_def : st2_def);
 }
 
+// Forward (gx NULL): in = x, out = t (may be NULL), scalar = loss (written).
+// Backward: in = t, out = gx, scalar = g (read).
+int loss_common(const float *weights, int nweights, int boundary, skel_handle in, skel_handle out, skel_handle scalar,
+                skel_handle gx, cudaStream_t s)
+{
+    if (!valid_handle(in) || (out && !valid_handle(out))) return fail(SKEL_ERR_INVALID_ARG, "bad handle");
+    if (in->ndim != 2) return fail(SKEL_ERR_UNSUPPORTED, "composed loss: 2D grids only");
+    if (in->dtype != SKEL_F32 || (out && out->dtype != SKEL_F32)) return fail(SKEL_ERR_DTYPE, "composed loss: float32 only");
+    if (out && (out->ndim != 2 || out->shape[0] != in->shape[0] || out->shape[1] != in->shape[1]))
+        return fail(SKEL_ERR_SHAPE, "composed loss: shapes differ");
+    if (boundary < SKEL_CLAMP || boundary > SKEL_PERIODIC) return fail(SKEL_ERR_INVALID_ARG, "unknown boundary");
+    if (weights && nweights != 9) return fail(SKEL_ERR_SHAPE, "2D weights: need 9 values (3x3 row-major)");
+    bool exact = false;
+    if ((out && device_overlap(in, out, &exact)) || device_overlap(in, scalar, &exact) ||
+        (out && device_overlap(out, scalar, &exact)))
+        return fail(SKEL_ERR_INVALID_ARG, "composed loss: operands overlap");
+    int rc = loss_fused_check(in->shape[0], in->shape[1], boundary);
+    if (rc) return rc;
+    std::vector<Operand> ops{{in, SKEL_READ}, {scalar, gx ? SKEL_READ : SKEL_WRITE}};
+    if (out) ops.push_back({out, SKEL_WRITE});
+    if ((rc = acquire_all(ops, s, nullptr))) return rc;
+    std::vector<float> wbuf;
+    LossLaunch l{};
+    l.boundary = boundary;
+    l.w = weights ? weights : default_weights(SKEL_FN_STENCIL9, 1, wbuf);
+    l.rows = in->shape[0];
+    l.cols = in->shape[1];
+    if (gx) {
+        l.t = static_cast<float *>(ops[0].ptr);
+        l.g = static_cast<const float *>(ops[1].ptr);
+        l.gx = static_cast<float *>(ops[2].ptr);
+    } else {
+        l.x = static_cast<const float *>(ops[0].ptr);
+        l.L = static_cast<float *>(ops[1].ptr);
+        l.t = out ? static_cast<float *>(ops[2].ptr) : nullptr;
+    }
+    return launch_loss(l, s);
+}
+
 }  // namespace
 
 extern "C" {
@@ -1113,6 +1152,27 @@ int skel_compose_map_stencil_sumsq(skel_fn map_fn, const double *params, int npa
         }, compose_default);
         if (rc) return rc;
         return result_host ? copy_result_to_host(result_host, out, 4, s) : (int)SKEL_OK;
+    });
+}
+
+int skel_composed_loss(const float *weights, int nweights, skel_boundary boundary, skel_handle x, skel_handle t,
+                       skel_handle loss, void *stream)
+{
+    return guarded([&] {
+        if (!valid_handle(loss) || loss->n != 1 || loss->dtype != SKEL_F32)
+            return fail(SKEL_ERR_SHAPE, "composed loss: loss must hold 1 float32 element");
+        return loss_common(weights, nweights, boundary, x, t, loss, nullptr, (cudaStream_t)stream);
+    });
+}
+
+int skel_composed_loss_bwd(const float *weights, int nweights, skel_boundary boundary, skel_handle t, skel_handle g,
+                           skel_handle gx, void *stream)
+{
+    return guarded([&] {
+        if (!valid_handle(g) || g->n != 1 || g->dtype != SKEL_F32)
+            return fail(SKEL_ERR_SHAPE, "composed loss: g must hold 1 float32 element");
+        if (!valid_handle(gx)) return fail(SKEL_ERR_INVALID_ARG, "bad handle");
+        return loss_common(weights, nweights, boundary, t, gx, g, gx, (cudaStream_t)stream);
     });
 }
 

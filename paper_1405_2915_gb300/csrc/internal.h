@@ -56,8 +56,10 @@ int kernel_occupancy(K kern, int threads, int dyn)
     for (const Entry &e : cache)
         if (e.k == reinterpret_cast<const void *>(kern) && e.dev == dev && e.threads == threads && e.dyn == dyn)
             return e.occ;
-    int occ = 0;
-    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, dyn);
+    int occ = 0, most = dyn;   // a kernel used with several sizes keeps the opt-in of the largest
+    for (const Entry &e : cache)
+        if (e.k == reinterpret_cast<const void *>(kern) && e.dev == dev && e.occ > 0 && e.dyn > most) most = e.dyn;
+    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, most);
     if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, kern, threads, dyn);
     if (e != cudaSuccess) {
         cudaGetLastError();
@@ -256,6 +258,21 @@ int launch_compose_fused(const ComposeLaunch &cl, const Choice &c, float *partia
 int compose_variant_count();
 const char *compose_variant_name(int v);
 Choice compose_default();
+
+// The composed loss (k_loss.cu): forward when gx is NULL (x -> t, L; t may
+// be NULL), else backward (t, g -> gx).
+struct LossLaunch {
+    int boundary;        // CLAMP or ZERO
+    const float *w;      // 9 weights, host copy
+    const float *x;
+    float *t;
+    float *L;            // 1 element
+    const float *g;      // 1 element, device
+    float *gx;
+    int64_t rows, cols;
+};
+int loss_fused_check(int64_t rows, int64_t cols, int boundary);
+int launch_loss(const LossLaunch &l, cudaStream_t s);
 
 // MapArray over a grid (fn COULOMB): atoms (m x 4 float32: x, y, z, q),
 // out rows x cols, grid position of out[i, j] = (j*h, i*h, z0).
