@@ -24,6 +24,8 @@ from ._lib import BOUNDARY, FN, SK, SkelError, F32, I32, I64, READ, WRITE, READW
 lib = _lib.load()
 
 _NP2DT = {np.dtype(np.float32): F32, np.dtype(np.int32): I32, np.dtype(np.int64): I64}
+_TORCH2DT = {}   # filled when torch is first needed
+_I64x2 = C.c_int64 * 2
 _DT2NP = {F32: np.float32, I32: np.int32, I64: np.int64}
 
 
@@ -32,22 +34,38 @@ def check(rc: int) -> None:
         raise SkelError(rc, lib.skel_last_error().decode())
 
 
+_torch_module = None
+
+
 def _torch():
-    import torch
-    return torch
+    global _torch_module
+    if _torch_module is None:
+        import torch
+        _torch_module = torch
+    return _torch_module
+
+
+_raw_stream = None   # torch's current stream of a device as an integer, once CUDA is initialised
 
 
 def current_stream() -> int:
     """cudaStream_t of torch's current stream (0 = legacy default stream)."""
-    return _torch().cuda.current_stream().cuda_stream
+    global _raw_stream
+    if _raw_stream is not None:
+        get, device = _raw_stream
+        return get(device())
+    torch = _torch()
+    s = torch.cuda.current_stream().cuda_stream   # initialises CUDA
+    get, device = (getattr(torch._C, n, None) for n in ("_cuda_getCurrentRawStream", "_cuda_getDevice"))
+    if get is not None and device is not None:
+        _raw_stream = (get, device)
+    return s
 
 
-def _stream(stream) -> C.c_void_p:
+def _stream(stream) -> int:
     if stream is None:
-        stream = current_stream()
-    elif not isinstance(stream, int):
-        stream = stream.cuda_stream
-    return C.c_void_p(stream)
+        return current_stream()
+    return stream if isinstance(stream, int) else stream.cuda_stream
 
 
 # ------------------------------------------------------------- allocator ---
@@ -90,6 +108,7 @@ class Container:
 
     def __init__(self, handle: int, keep=(), parent: "Container | None" = None):
         self.handle = C.c_void_p(handle)
+        self._h = handle             # the same as a plain integer (None once closed)
         self._keep = list(keep)
         self._parent = parent
         self._views = 0
@@ -111,13 +130,14 @@ class Container:
         torch = _torch()
         if not t.is_cuda or not t.is_contiguous():
             raise ValueError("from_tensor needs a contiguous CUDA tensor")
-        dt = {torch.float32: F32, torch.int32: I32, torch.int64: I64}[t.dtype]
-        shape = tuple(t.shape) if t.dim() in (1, 2) else (t.numel(),)
-        arr = (C.c_int64 * 2)(*shape, *([1] * (2 - len(shape))))
+        if not _TORCH2DT:
+            _TORCH2DT.update({torch.float32: F32, torch.int32: I32, torch.int64: I64})
+        dt = _TORCH2DT[t.dtype]
+        nd = t.dim()
+        arr = _I64x2(*t.shape) if nd == 2 else _I64x2(t.numel(), 1)
         h = C.c_void_p()
-        hp = None if host is None else host.ctypes.data
-        check(lib.skel_container_wrap(dt, len(shape), arr, C.c_void_p(hp), C.c_void_p(t.data_ptr()),
-                                      UNIT_DEVICE, C.byref(h)))
+        check(lib.skel_container_wrap(dt, 2 if nd == 2 else 1, arr, None if host is None else host.ctypes.data,
+                                      t.data_ptr(), UNIT_DEVICE, C.byref(h)))
         return cls(h.value, keep=[t] + ([host] if host is not None else []))
 
     @classmethod
@@ -189,7 +209,7 @@ class Container:
             check(lib.skel_container_destroy(self.handle))
             if self._parent is not None:
                 self._parent._views -= 1
-        self.handle = None
+        self.handle = self._h = None
         self._keep = []
 
     def __del__(self):
@@ -208,20 +228,28 @@ class Container:
         self.close()
 
 
+_HANDLES = [C.c_void_p * k for k in range(4)]
+
+
 def _handles(cs: Sequence[Container | None]):
-    arr = (C.c_void_p * max(1, len(cs)))()
-    for i, c in enumerate(cs):
-        arr[i] = None if c is None else c.handle.value
-    return arr
+    n = len(cs)
+    arr = _HANDLES[n] if 0 < n < 4 else C.c_void_p * max(1, n)
+    return arr(*[None if c is None else c._h for c in cs])
 
 
 def _fn(name) -> int:
     return name if isinstance(name, int) else FN[name]
 
 
+_DOUBLE1 = C.c_double * 1
+
+
 def _params(p):
-    p = list(p or [])
-    return (C.c_double * max(1, len(p)))(*p), len(p)
+    p = list(p) if p is not None else ()
+    n = len(p)
+    if n == 0:
+        return None, 0
+    return (_DOUBLE1 if n == 1 else C.c_double * n)(*p), n
 
 
 def _weights(w):
@@ -238,20 +266,18 @@ def skel_map(fn, ins: Sequence[Container], out: Container, params=(), stream=Non
 
 
 def skel_reduce(op, x: Container, result_dev: Container | None = None, host: bool = True, stream=None):
-    dt = x.info()[0]
-    res = np.zeros(1, dtype=dt)
-    check(lib.skel_reduce(_fn(op), x.handle, C.c_void_p(res.ctypes.data) if host else None,
+    res = C.c_uint32() if host else None   # the result's bits
+    check(lib.skel_reduce(_fn(op), x.handle, C.byref(res) if host else None,
                           None if result_dev is None else result_dev.handle, _stream(stream)))
-    return res[0] if host else None
+    return np.uint32(res.value).view(x.info()[0]) if host else None
 
 
 def skel_mapreduce(map_fn, red_op, ins: Sequence[Container], result_dev: Container | None = None,
                    host: bool = True, stream=None):
-    res = np.zeros(1, dtype=np.float32)
-    check(lib.skel_mapreduce(_fn(map_fn), _fn(red_op), _handles(ins), len(ins),
-                             C.c_void_p(res.ctypes.data) if host else None,
+    res = C.c_uint32() if host else None
+    check(lib.skel_mapreduce(_fn(map_fn), _fn(red_op), _handles(ins), len(ins), C.byref(res) if host else None,
                              None if result_dev is None else result_dev.handle, _stream(stream)))
-    return res[0] if host else None
+    return np.uint32(res.value).view(np.float32) if host else None
 
 
 def skel_scan(op, inclusive: bool, x: Container, out: Container, stream=None) -> None:
@@ -288,14 +314,14 @@ def skel_compose_map_stencil_sumsq(map_fn, stencil, x: Container, params=(), wei
                                    result_dev: Container | None = None, host: bool = True, stream=None):
     """sum_{i,j} (S map_fn(x))[i,j]^2 as one composed call (Map -> 2D
     MapOverlap -> MapReduce); returns the value when host is True."""
-    res = np.zeros(1, dtype=np.float32)
+    res = C.c_uint32() if host else None
     p, np_ = _params(params)
     w = _weights(weights)
     check(lib.skel_compose_map_stencil_sumsq(_fn(map_fn), p, np_, _fn(stencil), w[0], w[1],
                                              BOUNDARY[boundary] if isinstance(boundary, str) else boundary, x.handle,
-                                             C.c_void_p(res.ctypes.data) if host else None,
+                                             C.byref(res) if host else None,
                                              None if result_dev is None else result_dev.handle, _stream(stream)))
-    return res[0] if host else None
+    return np.uint32(res.value).view(np.float32) if host else None
 
 
 def skel_composed_loss(weights, boundary, x: Container, t: Container | None, loss: Container, stream=None) -> None:

@@ -488,6 +488,40 @@ int copy_result_to_host(void *dst, const void *src_dev, size_t bytes, cudaStream
     return SKEL_OK;
 }
 
+// Where a scalar call leaves its result: the caller's container; else, for a
+// result only the host reads, a pinned slot the kernel writes directly (a
+// pageable 4-byte copy behind the kernel cost another 10 us); else the
+// stream's device slot.
+struct ScalarResult {
+    void *out = nullptr;
+    HostSlot *slot = nullptr;
+    int open(void *dev, cudaStream_t s)
+    {
+        if (dev) {
+            out = dev;
+            return SKEL_OK;
+        }
+        slot = new (buf) HostSlot();
+        if (slot->index >= 0) {
+            out = slot->dev;
+            return SKEL_OK;
+        }
+        return result_slot(s, &out);
+    }
+    int read(void *dst, size_t bytes, cudaStream_t s)
+    {
+        if (!slot || slot->index < 0) return copy_result_to_host(dst, out, bytes, s);
+        SKEL_CUDA_TRY(cudaStreamSynchronize(s));
+        std::memcpy(dst, slot->host, bytes);
+        return SKEL_OK;
+    }
+    ~ScalarResult()
+    {
+        if (slot) slot->~HostSlot();
+    }
+    alignas(HostSlot) unsigned char buf[sizeof(HostSlot)];
+};
+
 Choice reduce_def() { return reduce_default(); }
 Choice map_def() { return map_default(); }
 Choice scan_def() { return scan_default(); }
@@ -771,14 +805,13 @@ int reduce_common(int sk, int map_fn, int op, const skel_handle *ins, int nin, v
     int res = 0;
     int rc = acquire_all(ops, s, &res);
     if (rc) return rc;
-    void *out = nullptr;
-    if (result_dev) out = ops.back().ptr;
-    else if ((rc = result_slot(s, &out))) return rc;
-    ReduceLaunch r{op, map_fn, dt, ops[0].ptr, nin == 2 ? ops[1].ptr : nullptr, out, ins[0]->n};
+    ScalarResult res1;
+    if ((rc = res1.open(result_dev ? ops.back().ptr : nullptr, s))) return rc;
+    ReduceLaunch r{op, map_fn, dt, ops[0].ptr, nin == 2 ? ops[1].ptr : nullptr, res1.out, ins[0]->n};
     Context ctx{sk, sk == SKEL_SK_MAPREDUCE ? map_fn : op, dt, ins[0]->n, 0, res};
     rc = run_with_fallback(sk, ctx, [&](const Choice &c) { return launch_reduce(r, c, s); }, reduce_def);
     if (rc) return rc;
-    if (result_host) return copy_result_to_host(result_host, out, 4, s);
+    if (result_host) return res1.read(result_host, 4, s);
     return SKEL_OK;
 }
 
@@ -1086,9 +1119,9 @@ int skel_compose_map_stencil_sumsq(skel_fn map_fn, const double *params, int npa
         int res = 0;
         int rc = acquire_all(ops, s, &res);
         if (rc) return rc;
-        void *out = nullptr;
-        if (result_dev) out = ops.back().ptr;
-        else if ((rc = result_slot(s, &out))) return rc;
+        ScalarResult res1;
+        if ((rc = res1.open(result_dev ? ops.back().ptr : nullptr, s))) return rc;
+        void *out = res1.out;
         const int64_t n = in->n;
         std::vector<float> wbuf;
         ComposeLaunch cl{map_fn, map_fn == SKEL_FN_SCALE ? (float)params[0] : 0.f, boundary,
@@ -1104,7 +1137,7 @@ int skel_compose_map_stencil_sumsq(skel_fn map_fn, const double *params, int npa
         };
         if (n == 0) {   // the empty sum: 0
             if ((rc = sumsq(nullptr, 0, SKEL_FN_SQ))) return rc;
-            return result_host ? copy_result_to_host(result_host, out, 4, s) : (int)SKEL_OK;
+            return result_host ? res1.read(result_host, 4, s) : (int)SKEL_OK;
         }
         Context ctx{SKEL_SK_COMPOSE, stencil, SKEL_F32, n, 1, res};
         rc = run_with_fallback(SKEL_SK_COMPOSE, ctx, [&](const Choice &c) -> int {
@@ -1151,7 +1184,7 @@ int skel_compose_map_stencil_sumsq(skel_fn map_fn, const double *params, int npa
             return r1;
         }, compose_default);
         if (rc) return rc;
-        return result_host ? copy_result_to_host(result_host, out, 4, s) : (int)SKEL_OK;
+        return result_host ? res1.read(result_host, 4, s) : (int)SKEL_OK;
     });
 }
 

@@ -116,6 +116,17 @@ int noalloc_take_status(uint32_t *err);
 // Fixed 256-byte device buffer of `stream` for scalar results.
 int result_slot(cudaStream_t stream, void **out);
 
+// A pinned host slot of 4 bytes that kernels can write (dev) and the caller
+// reads (host) once the stream is done; index < 0: none was free.
+struct HostSlot {
+    int index = -1;
+    void *host = nullptr, *dev = nullptr;
+    HostSlot();
+    ~HostSlot();
+    HostSlot(const HostSlot &) = delete;
+    HostSlot &operator=(const HostSlot &) = delete;
+};
+
 // Allocation through the active allocator; free_dev must be given the same
 // allocator record that allocated.
 struct Allocator {

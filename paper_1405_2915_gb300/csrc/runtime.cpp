@@ -225,6 +225,51 @@ int result_slot(cudaStream_t stream, void **out)
     return SKEL_OK;
 }
 
+// Pinned 4-byte slots that a kernel writes a scalar result into when the
+// caller reads it on the host: the call then only waits for its stream,
+// without a copy behind the kernel.  One page for the process, a slot per
+// call in flight; more than kHostSlots calls at once use the copy instead.
+namespace {
+constexpr int kHostSlots = 64, kHostSlotBytes = 64;
+std::mutex g_hslot_mu;
+unsigned char *g_hslot_host = nullptr, *g_hslot_dev = nullptr;
+uint64_t g_hslot_used = 0;
+}  // namespace
+
+HostSlot::HostSlot()
+{
+    std::lock_guard<std::mutex> lk(g_hslot_mu);
+    if (!g_hslot_host) {
+        void *h = nullptr, *d = nullptr;
+        if (cudaHostAlloc(&h, kHostSlots * kHostSlotBytes, cudaHostAllocPortable | cudaHostAllocMapped) != cudaSuccess) {
+            cudaGetLastError();
+            return;
+        }
+        if (cudaHostGetDevicePointer(&d, h, 0) != cudaSuccess) {
+            cudaGetLastError();
+            cudaFreeHost(h);
+            return;
+        }
+        g_hslot_host = static_cast<unsigned char *>(h);
+        g_hslot_dev = static_cast<unsigned char *>(d);
+    }
+    for (int k = 0; k < kHostSlots; ++k)
+        if (!(g_hslot_used >> k & 1)) {
+            g_hslot_used |= uint64_t(1) << k;
+            index = k;
+            host = g_hslot_host + k * kHostSlotBytes;
+            dev = g_hslot_dev + k * kHostSlotBytes;
+            return;
+        }
+}
+
+HostSlot::~HostSlot()
+{
+    if (index < 0) return;
+    std::lock_guard<std::mutex> lk(g_hslot_mu);
+    g_hslot_used &= ~(uint64_t(1) << index);
+}
+
 // Device-side status words of the scratch of `stream` (current device), or
 // nullptr if the stream never used scratch.
 Control *scratch_control(cudaStream_t stream)
@@ -257,6 +302,13 @@ int release_scratch()
     cudaSetDevice(cur);
     g_scratch.clear();
     g_slots.clear();
+    {
+        std::lock_guard<std::mutex> lh(g_hslot_mu);
+        if (g_hslot_host && !g_hslot_used) {   // no call waits on a slot
+            cudaFreeHost(g_hslot_host);
+            g_hslot_host = g_hslot_dev = nullptr;
+        }
+    }
     std::lock_guard<std::mutex> lp(g_pool_mu);
     for (cudaMemPool_t pool : g_pool)
         if (pool) cudaMemPoolTrimTo(pool, 0);   // memory no allocation holds goes back
