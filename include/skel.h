@@ -329,11 +329,11 @@ int skel_mapoverlap_chain(skel_fn fn, const float *weights, int nweights, skel_b
  * Table key (SKEL_SK_COMPOSE, stencil, F32, n, radius 1, residency).
  * Variants: per_call (the Map, MapOverlap and MapReduce calls, each
  * dispatched as usual, through two n-element temporaries: 20 bytes of HBM
- * traffic per point) and fused (tile 0..2: 32 << tile rows per block; one
- * pass reading in once, 4 bytes per point, then one Reduce of the block
- * partials; needs 16-byte aligned rows, cols % 4 == 0).  Both compute every
- * stencil output with the same float32 operations; the sums differ in
- * order only.  n = 0 gives 0. */
+ * traffic per point), fused (one launch reading in once, 4 bytes per point;
+ * tile 0..2: one wave of 32, 24 or 16 warps per SM; needs 16-byte aligned
+ * rows, cols % 4 == 0) and fused_any (the same for any alignment and width).
+ * All compute every stencil output with the same float32 operations; the
+ * sums differ in order only.  n = 0 gives 0. */
 int skel_compose_map_stencil_sumsq(skel_fn map_fn, const double *params, int nparams, skel_fn stencil,
                                    const float *weights, int nweights, skel_boundary boundary, skel_handle in,
                                    void *result_host, skel_handle result_dev, void *stream);

@@ -1141,17 +1141,7 @@ int skel_compose_map_stencil_sumsq(skel_fn map_fn, const double *params, int npa
         }
         Context ctx{SKEL_SK_COMPOSE, stencil, SKEL_F32, n, 1, res};
         rc = run_with_fallback(SKEL_SK_COMPOSE, ctx, [&](const Choice &c) -> int {
-            if (c.variant == 1) {
-                int64_t np = 0;
-                int r1 = compose_fused_check(cl, c, &np);
-                if (r1) return r1;
-                float *parts = static_cast<float *>(dev_alloc(rec, (size_t)np * 4, s));
-                if (!parts) return fail(SKEL_ERR_OOM, "composed chain: partial sums");
-                r1 = launch_compose_fused(cl, c, parts, s);
-                if (!r1) r1 = sumsq(parts, np, -1);
-                dev_free(rec, parts, s);
-                return r1;
-            }
+            if (c.variant == 1 || c.variant == 2) return launch_compose_fused(cl, c, static_cast<float *>(out), s);
             if (c.variant != 0) return fail(SKEL_ERR_INVALID_ARG, "composed chain: unknown variant");
             // per call: Map -> MapOverlap -> MapReduce(sq, +), each dispatched
             float *t = static_cast<float *>(dev_alloc(rec, (size_t)n * 4, s));

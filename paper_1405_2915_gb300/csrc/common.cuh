@@ -67,6 +67,33 @@ __device__ __forceinline__ uint64_t globaltimer()
     return t;
 }
 
+// Asynchronous copies into shared memory (16 bytes bypass L1; 4 bytes for
+// rows of any alignment), in groups that are waited for in order.
+__device__ __forceinline__ void cp_async16(uint32_t dst, const float *src)
+{
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" :: "r"(dst), "l"(src) : "memory");
+}
+__device__ __forceinline__ void cp_async4(uint32_t dst, const float *src)
+{
+    asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" :: "r"(dst), "l"(src) : "memory");
+}
+__device__ __forceinline__ void cp_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
+template <int N>
+__device__ __forceinline__ void cp_wait() { asm volatile("cp.async.wait_group %0;" :: "n"(N) : "memory"); }
+
+// A float32 sum and the rounding errors it made, each exact (Knuth's TwoSum).
+struct Sum2 {
+    float hi = 0.f, lo = 0.f;
+    __device__ __forceinline__ void add(float v)
+    {
+        const float s = hi + v, bv = s - hi;
+        lo += (hi - (s - bv)) + (v - bv);
+        hi = s;
+    }
+    // an infinite sum has no meaningful error term
+    __device__ __forceinline__ double value() const { return isinf(hi) ? (double)hi : (double)hi + (double)lo; }
+};
+
 // The first statement of every kernel.  launch_kernel lets a kernel's blocks
 // be set up while the stream's previous kernel drains (programmatic dependent
 // launch); this waits until that kernel has completed and its writes are

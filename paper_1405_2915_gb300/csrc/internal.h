@@ -253,7 +253,7 @@ const char *stencil_variant_name(int ndim, int v);
 Choice stencil_default(int ndim);
 
 // The composed chain Map -> MapOverlap (2D, radius 1) -> MapReduce(sq, +),
-// fused into one pass over x (variant 1 of SKEL_SK_COMPOSE).
+// fused into one pass over x (variants 1 and 2 of SKEL_SK_COMPOSE).
 struct ComposeLaunch {
     int map_fn;          // SKEL_FN_TANH / SQ / SCALE / COPY
     float a;             // the map's parameter (SCALE)
@@ -263,9 +263,7 @@ struct ComposeLaunch {
     const float *in;
     int64_t rows, cols;
 };
-// Checks the fused variant's constraints; *nparts: the partial sums it writes.
-int compose_fused_check(const ComposeLaunch &cl, const Choice &c, int64_t *nparts);
-int launch_compose_fused(const ComposeLaunch &cl, const Choice &c, float *partials, cudaStream_t s);
+int launch_compose_fused(const ComposeLaunch &cl, const Choice &c, float *out, cudaStream_t s);
 int compose_variant_count();
 const char *compose_variant_name(int v);
 Choice compose_default();

@@ -48,18 +48,6 @@ constexpr int kLMaxCols = 8192;
 constexpr int kLWarps = 32;                   // most warps of a block
 constexpr int kFwdRing = 4, kBwdRing = 6;     // rows in shared memory; 3 of them in flight
 
-__device__ __forceinline__ void cp_async16(uint32_t dst, const float *src)
-{
-    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" :: "r"(dst), "l"(src) : "memory");
-}
-__device__ __forceinline__ void cp_async4(uint32_t dst, const float *src)
-{
-    asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" :: "r"(dst), "l"(src) : "memory");
-}
-__device__ __forceinline__ void cp_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
-template <int N>
-__device__ __forceinline__ void cp_wait() { asm volatile("cp.async.wait_group %0;" :: "n"(N) : "memory"); }
-
 // Floats of one ring row of `threads` threads with C columns each: C / 4
 // planes of 4 floats per thread, each plane 32 / (C / 4) floats longer so that
 // 4-byte copies of 32 consecutive columns meet no bank twice.
@@ -128,19 +116,6 @@ __device__ __forceinline__ double warp_sum(double v)
     return v;
 }
 
-// A float32 sum and the rounding errors it made, each exact (Knuth's TwoSum).
-struct Sum2 {
-    float hi = 0.f, lo = 0.f;
-    __device__ __forceinline__ void add(float v)
-    {
-        const float s = hi + v, bv = s - hi;
-        lo += (hi - (s - bv)) + (v - bv);
-        hi = s;
-    }
-    // an infinite sum has no meaningful error term
-    __device__ __forceinline__ double value() const { return isinf(hi) ? (double)hi : (double)hi + (double)lo; }
-};
-
 // The part of a thread's work both directions share: its columns, the ring,
 // the edges of the row.
 template <bool VEC, int C>
@@ -195,19 +170,19 @@ struct RowStream {
 #pragma unroll
                 for (int m = 0; m < NP; ++m) {  // group q of four columns: plane q % NP, thread q / NP
                     const int q = m * nthr + threadIdx.x;
-                    if (4 * q < cols) cp_async16(d + (uint32_t)((q % NP) * pf + (q / NP) * 4) * 4u, next + 4 * q);
+                    if (4 * q < cols) dev::cp_async16(d + (uint32_t)((q % NP) * pf + (q / NP) * 4) * 4u, next + 4 * q);
                 }
             } else {
 #pragma unroll
                 for (int m = 0; m < C; ++m) {
                     const int e = m * nthr + threadIdx.x;
-                    if (e < cols) cp_async4(d + (uint32_t)((e / 4 % NP) * pf + (e / C) * 4 + e % 4) * 4u, next + e);
+                    if (e < cols) dev::cp_async4(d + (uint32_t)((e / 4 % NP) * pf + (e / C) * 4 + e % 4) * 4u, next + e);
                 }
             }
             next += cols;
             ++ncopied;
         }
-        cp_commit();
+        dev::cp_commit();
     }
     __device__ __forceinline__ void read(int i, float (&v)[C]) const
     {
@@ -303,16 +278,16 @@ loss_fwd(const float *__restrict__ x, float *__restrict__ t_out, int64_t rows, i
     const int nin = (int)((bottom ? rows : r1 + 1) - q0);
     RowStream<VEC, C> rs(x, rows, cols, q0, nin, dyn, kFwdRing);
     const int lane = rs.lane, warp = rs.warp;
-    Sum2 su, ss;
+    dev::Sum2 su, ss;
     float P1[C], P2[C];
 #pragma unroll
     for (int j = 0; j < C; ++j) P1[j] = P2[j] = 0.f;
 #pragma unroll
     for (int k = 0; k < kFwdRing - 1; ++k) rs.copy_next();
-    cp_wait<kFwdRing - 2>();
+    dev::cp_wait<kFwdRing - 2>();
     __syncthreads();
 
-    auto sum_sq = [&](float (&o)[C], Sum2 &k) {   // the grid's columns only
+    auto sum_sq = [&](float (&o)[C], dev::Sum2 &k) {   // the grid's columns only
         rs.mask(o);
         float q[4] = {0.f, 0.f, 0.f, 0.f};
 #pragma unroll
@@ -343,7 +318,7 @@ loss_fwd(const float *__restrict__ x, float *__restrict__ t_out, int64_t rows, i
             exi.last[warp] = v[C - 1];
             exi.total[warp] = wi;
         }
-        cp_wait<kFwdRing - 3>();   // row i + 1 has landed (its copies by every thread, after the barrier)
+        dev::cp_wait<kFwdRing - 3>();   // row i + 1 has landed (its copies by every thread, after the barrier)
         __syncthreads();
         rs.copy_next();            // into the slot of row i - 1
         neighbours(v, exi, lane, warp, rs.nwarps, e);
@@ -375,7 +350,7 @@ loss_fwd(const float *__restrict__ x, float *__restrict__ t_out, int64_t rows, i
         add_row(w, mid, e, P1, P2, o);
         sum_sq(o, su);
     }
-    cp_wait<0>();
+    dev::cp_wait<0>();
     double a = warp_sum(su.value()), c = warp_sum(ss.value());
     if (lane == 0) red[warp] = make_double2(a, c);
     __syncthreads();
@@ -434,7 +409,7 @@ loss_bwd(const float *__restrict__ t, const float *__restrict__ g, float *__rest
     float L1 = 0.f, L2 = 0.f, R1 = 0.f, R2 = 0.f;   // the columns beside the grid (below)
 #pragma unroll
     for (int k = 0; k < 3; ++k) rs.copy_next();
-    cp_wait<2>();
+    dev::cp_wait<2>();
     __syncthreads();
 
     for (int i = 0; i < niter; ++i) {
@@ -499,7 +474,7 @@ loss_bwd(const float *__restrict__ t, const float *__restrict__ g, float *__rest
             ex[1].total[warp] = rwi;
         }
         if (lane == 31) ex[1].last[warp] = u[C - 1];
-        cp_wait<2>();                         // row i + 1 has landed (visible after the barrier)
+        dev::cp_wait<2>();                         // row i + 1 has landed (visible after the barrier)
         __syncthreads();
         // ---- phase 3: the adjoint stencil of row - 2, gx of row - 2 ----
         neighbours(u, ex[1], lane, warp, rs.nwarps, e);    // 0 outside the grid
@@ -542,7 +517,7 @@ loss_bwd(const float *__restrict__ t, const float *__restrict__ g, float *__rest
             rs.write(i - 2, y, gx + (row - 2) * cols);
         }
     }
-    cp_wait<0>();
+    dev::cp_wait<0>();
 }
 
 // Threads of a block with C columns each: whole warps.

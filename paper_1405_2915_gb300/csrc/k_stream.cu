@@ -49,30 +49,15 @@ namespace skel {
 namespace {
 
 constexpr int kStreamWarps = 4;   // warps per block
-constexpr int kStreamCols = 128;  // columns of a strip, 4 per lane
-constexpr int kStreamRing = 8;    // input rows in flight per warp (4 KiB)
 
 template <int K>
 struct StreamGeom {
     static constexpr int HL = (K + 3) / 4 * 4;           // halo columns on each side, whole lanes
-    static constexpr int W = kStreamCols - 2 * HL;       // output columns per strip
+    static constexpr int W = kStripCols - 2 * HL;       // output columns per strip
     // rows of shared memory per warp: the ring, a held row per stage, a row being stored
-    static constexpr int rows = kStreamRing + K + 1;
-    static constexpr int smem_bytes = kStreamWarps * rows * kStreamCols * 4;
+    static constexpr int rows = kStripRing + K + 1;
+    static constexpr int smem_bytes = kStreamWarps * rows * kStripCols * 4;
 };
-
-__device__ __forceinline__ void cp_async16(uint32_t dst, const float *src)
-{
-    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" :: "r"(dst), "l"(src) : "memory");
-}
-__device__ __forceinline__ void cp_async4(uint32_t dst, const float *src)
-{
-    asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" :: "r"(dst), "l"(src) : "memory");
-}
-__device__ __forceinline__ void cp_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
-
-template <int N>
-__device__ __forceinline__ void cp_wait() { asm volatile("cp.async.wait_group %0;" :: "n"(N) : "memory"); }
 
 // VEC: rows start on 16-byte boundaries (in, out aligned, cols % 4 == 0).
 // H: output rows per segment; strips: strips per row of the grid; nwork:
@@ -84,8 +69,7 @@ st2_stream(const float *__restrict__ in, float *__restrict__ out, int64_t rows, 
 {
     dev::grid_wait();
     using G = StreamGeom<K>;
-    constexpr int C = 4, SW = kStreamCols, RING = kStreamRing;
-    constexpr uint32_t RB = SW * 4;                     // bytes of a ring row
+    constexpr int C = 4, SW = kStripCols, RING = kStripRing;
     extern __shared__ __align__(16) float sm[];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int64_t gw = (int64_t)blockIdx.x * kStreamWarps + warp;
@@ -110,43 +94,8 @@ st2_stream(const float *__restrict__ in, float *__restrict__ out, int64_t rows, 
     const bool lead = !wrap && c0 == 0, trail = !wrap && c0 + C >= cols;
     const int nv = trail ? (int)(cols - c0) : C;        // grid columns of the lane (<= 0: none)
 
-    // ---- the ring: row q0 + i goes to slot i % RING ----
-    constexpr int NL = VEC ? 1 : 4;                     // copies per lane and row
-    const uint32_t ring_s = (uint32_t)__cvta_generic_to_shared(ring);
-    int64_t lrow = q0;
-    if (wrap) { lrow %= rows; if (lrow < 0) lrow += rows; }
-    // load index at which the rows wrap (PERIODIC)
-    int64_t wrap_at = wrap ? rows - lrow : INT64_MAX;
-    const float *src[NL];
-    bool ok[NL];
-#pragma unroll
-    for (int k = 0; k < NL; ++k) {
-        int64_t c = VEC ? g0 + 4 * (32 * k + lane) : g0 + 32 * k + lane;
-        if (wrap) { c %= cols; if (c < 0) c += cols; }
-        ok[k] = c >= 0 && c < cols;
-        src[k] = in + lrow * cols + (ok[k] ? c : 0);
-    }
-    auto issue = [&](int i) {
-        if (i < nin) {
-            const uint32_t d = ring_s + (uint32_t)(i & (RING - 1)) * RB;
-            if (i == wrap_at) {
-                wrap_at += rows;
-#pragma unroll
-                for (int k = 0; k < NL; ++k) src[k] -= rows * cols;
-            }
-#pragma unroll
-            for (int k = 0; k < NL; ++k) {
-                if (ok[k]) {
-                    if (VEC) cp_async16(d + 16u * (32 * k + lane), src[k]);
-                    else cp_async4(d + 4u * (32 * k + lane), src[k]);
-                }
-                src[k] += cols;
-            }
-        }
-        cp_commit();
-    };
-#pragma unroll
-    for (int i = 0; i < RING - 1; ++i) issue(i);
+    StripRing<VEC> rows_in(in, rows, cols, wrap, q0, g0, nin, ring);
+    rows_in.start();
 
     float P1[K][C], P2[K][C];
 #pragma unroll
@@ -176,11 +125,11 @@ st2_stream(const float *__restrict__ in, float *__restrict__ out, int64_t rows, 
         constexpr bool ROWE = decltype(rowe_t)::value, COLE = decltype(cole_t)::value;
 #pragma unroll 1
         for (int i = i0; i < i1; ++i) {
-            cp_wait<RING - 2>();
+            dev::cp_wait<RING - 2>();
             __syncwarp();   // the row has landed for every lane; the last row's readers are done
             const float4 q = *reinterpret_cast<const float4 *>(ring + (i & (RING - 1)) * SW + C * lane);
             float x[C] = {q.x, q.y, q.z, q.w};
-            issue(i + RING - 1);
+            rows_in.copy(i + RING - 1);
 #pragma unroll
             for (int s = 0; s < K; ++s) {
                 if (ROWE) {
@@ -247,7 +196,7 @@ st2_stream(const float *__restrict__ in, float *__restrict__ out, int64_t rows, 
         else if (cedge) walk(i0, i1, F{}, T{});
         else walk(i0, i1, F{}, F{});
     }
-    cp_wait<0>();
+    dev::cp_wait<0>();
 }
 
 // Rows per segment: one wave of kStreamFill warps per SM, so that the 2K

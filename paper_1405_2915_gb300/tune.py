@@ -115,8 +115,9 @@ def candidates(sk_name: str):
             yield (1, 256, 0, k)
     elif sk_name == "compose":
         yield (0, 0, 0, 0)
-        for t in (0, 1, 2):      # fused: 32, 64, 128 rows per block
+        for t in (0, 1, 2):      # fused: one wave of 32, 24, 16 warps per SM; 2 takes rows of any alignment
             yield (1, 0, 0, t)
+            yield (2, 0, 0, t)
     elif sk_name == "edge":
         yield (0, 0, 0, 0)
         for t in (0, 1, 2):      # chunks of 8, 32, 128 MiB
