@@ -446,8 +446,10 @@ bool device_overlap(skel_handle a, skel_handle b, bool *exact)
     return o;
 }
 
-template <class Launch>
-int run_with_fallback(int sk, const Context &ctx, Launch launch, Choice (*def)())
+struct NoRule { void operator()(Choice &, bool) const {} };
+
+template <class Launch, class Rule = NoRule>
+int run_with_fallback(int sk, const Context &ctx, Launch launch, Choice (*def)(), Rule rule = Rule{})
 {
     // Selectability (conditional composition): a variant whose constraint
     // fails for this call reports SKEL_ERR_UNSUPPORTED; the call then falls
@@ -455,6 +457,7 @@ int run_with_fallback(int sk, const Context &ctx, Launch launch, Choice (*def)()
     // skeleton implements without constraints.
     bool forced = false;
     Choice c = select_variant(ctx, &forced);
+    rule(c, forced);   // what the table's key does not show
     int rc = launch(c);
     if (rc == SKEL_ERR_UNSUPPORTED && !forced) {
         const Choice fallbacks[2] = {def(), Choice{0, 0, 0, 0}};
@@ -521,6 +524,29 @@ struct ScalarResult {
     }
     alignas(HostSlot) unsigned char buf[sizeof(HostSlot)];
 };
+
+Choice scan_def();
+
+// A scan's variant.  The table is keyed by the total size alone; two rules
+// add what it cannot see.  Rows: one block per row (variant 9) wherever a row
+// fits a block's shared memory and either there is a row for every second SM
+// or a row is short (4097 x 4099 38 us against 298, 8192 x 256 9 against 96,
+// 4096 x 4096 29 against 33, 8192 x 8192 the same; 20 x 50000 11.5 against
+// 7.3, so few long rows take the look-back variants).  One sequence: the
+// table's variant 9 fits about 8.4 million elements; beyond, the same entry's
+// `tile` is the shape of variant 8.
+int dispatch_scan(const ScanLaunch &sc, const Context &ctx, cudaStream_t s)
+{
+    return run_with_fallback(SKEL_SK_SCAN, ctx, [&](const Choice &c) { return launch_scan(sc, c, s); }, scan_def,
+                             [&](Choice &c, bool forced) {
+                                 if (forced) return;
+                                 const bool fits = scan_wave_fits(sc), rows = sc.seg > 0 && sc.seg < sc.n;
+                                 if (rows && fits && (sc.seg <= 8192 || sc.n / sc.seg >= device_info().sms / 2))
+                                     c = Choice{9, 256, 4, 0};
+                                 else if (c.variant == 9 && (rows || !fits))   // variant 4 below 2^20 elements
+                                     c = sc.n < (1 << 20) ? Choice{4, 256, 4, 0} : Choice{8, 256, 4, c.tile};
+                             });
+}
 
 Choice reduce_def() { return reduce_default(); }
 Choice map_def() { return map_default(); }
@@ -1017,7 +1043,7 @@ int skel_scan(skel_fn op, int inclusive, skel_handle in, skel_handle out, void *
         // launch, so the work, not the row length, decides which is fastest
         // (a row length of 8192 once picked the one-block variant for 8192 rows)
         Context ctx{SKEL_SK_SCAN, inclusive ? 1 : 0, in->dtype, in->n, 0, res};
-        return run_with_fallback(SKEL_SK_SCAN, ctx, [&](const Choice &c) { return launch_scan(sc, c, s); }, scan_def);
+        return dispatch_scan(sc, ctx, s);
     });
 }
 
@@ -1563,7 +1589,7 @@ int skel_scan_bwd(skel_fn op, int inclusive, skel_handle gout, skel_handle gin, 
                       gout->ndim == 2 ? gout->shape[1] : 0};
         // reverse scans have their own keys (fn 2: exclusive, 3: inclusive)
         Context ctx{SKEL_SK_SCAN, inclusive ? 3 : 2, SKEL_F32, gout->n, 0, res};   // total work, as forward
-        return run_with_fallback(SKEL_SK_SCAN, ctx, [&](const Choice &c) { return launch_scan(sc, c, s); }, scan_def);
+        return dispatch_scan(sc, ctx, s);
     });
 }
 

@@ -224,6 +224,8 @@ struct ScanLaunch {
 };
 int launch_scan(const ScanLaunch &sc, const Choice &c, cudaStream_t s);
 int scan_rr_launch(const ScanLaunch &sc, const Choice &c, cudaStream_t s);   // variant 8 (k_scan_rr.cu)
+int scan_wave_launch(const ScanLaunch &sc, cudaStream_t s);   // variant 9 (k_scan_wave.cu)
+bool scan_wave_fits(const ScanLaunch &sc);
 int scan_variant_count();
 const char *scan_variant_name(int v);
 Choice scan_default();

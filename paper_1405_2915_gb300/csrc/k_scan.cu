@@ -39,6 +39,10 @@
 //                       publish their aggregates, scanner warps re-read
 //                       each tile from L2 during its look-back (k_scan_rr.cu;
 //                       same operand rules as variant 5).
+//   9 one_wave          one block per SM, each with its whole chunk in shared
+//                       memory and one exchange of the chunks' sums; rows:
+//                       one block per row (k_scan_wave.cu; any alignment, up
+//                       to 55296 elements per SM or row).
 //   6 lookback_ws       one persistent block per SM split into producer,
 //                       scanner, look-back and store warps that pass tiles
 //                       through a ring of staged tiles (tile=0: four 48 KiB
@@ -1568,22 +1572,23 @@ int run_scan_v(const ScanLaunch &sc, const Choice &c, cudaStream_t s)
 
 }  // namespace
 
-int scan_variant_count() { return 9; }
+int scan_variant_count() { return 10; }
 const char *scan_variant_name(int v)
 {
     static const char *names[] = {"reduce_then_scan", "lookback", "one_block", "lookback_block", "lookback_tma",
-                                  "lookback_big", "lookback_ws", "lookback_hybrid", "lookback_reread"};
-    return v >= 0 && v < 9 ? names[v] : "?";
+                                  "lookback_big", "lookback_ws", "lookback_hybrid", "lookback_reread", "one_wave"};
+    return v >= 0 && v < 10 ? names[v] : "?";
 }
 Choice scan_default() { return Choice{0, 256, 4, 0}; }
 
 int launch_scan(const ScanLaunch &sc, const Choice &c, cudaStream_t s)
 {
     if (sc.n == 0) return SKEL_OK;
-    if (c.variant < 0 || c.variant > 8) return fail(SKEL_ERR_INVALID_ARG, "scan: unknown variant");
+    if (c.variant < 0 || c.variant > 9) return fail(SKEL_ERR_INVALID_ARG, "scan: unknown variant");
     if (c.block > 0 && c.block != kBlock) return fail(SKEL_ERR_INVALID_ARG, "scan: block must be 256");
     if (sc.seg > 0 && sc.n % sc.seg) return fail(SKEL_ERR_SHAPE, "scan: n is not a multiple of the segment");
     if (c.variant == 8) return scan_rr_launch(sc, c, s);
+    if (c.variant == 9) return scan_wave_launch(sc, s);
     if (sc.dtype == SKEL_F32)
         return sc.inclusive ? run_scan_v<float, true>(sc, c, s) : run_scan_v<float, false>(sc, c, s);
     if (sc.dtype == SKEL_I32)

@@ -94,6 +94,7 @@ def candidates(sk_name: str):
             yield (7, 256, 4, t)
         for t in (0, 1, 2, 3):   # aggregators and re-reading scanners: ring tiles + scanners 6 + 6, 4 + 8, 6 + 8, 5 + 8
             yield (8, 256, 4, t)
+        yield (9, 256, 4, 0)     # one wave of blocks, chunks in shared memory
     elif sk_name == "mapoverlap2d":
         yield (0, 256, 0, 0)
         yield (1, 256, 0, 0)
