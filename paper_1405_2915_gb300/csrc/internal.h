@@ -83,7 +83,8 @@ struct Control {
     uint32_t queue;      // work queue of persistent kernels
     uint32_t exited;     // persistent blocks that left the work loop
     uint32_t epoch;      // last look-back tag of a kernel that keeps its tag on the device (0: none yet)
-    uint32_t pad[57];
+    uint32_t reject;     // a call's device-resident input failed validation (reset by that call's last kernel)
+    uint32_t pad[56];
 };
 static_assert(sizeof(Control) == 256, "control block is 256 bytes");
 constexpr uint32_t kErrTimeout = 1u;   // a bounded wait gave up
@@ -246,6 +247,9 @@ int launch_stencil(const StencilLaunch &st, const Choice &c, cudaStream_t s);
 // per pass (ping-pong between st.out and tmp, the last pass writes st.out).
 int launch_stream2d(bool taps5, int k, const float *in, float *out, int64_t rows, int64_t cols, int b, const float *w9,
                     cudaStream_t s);   // k steps in one pass (k_stream.cu)
+// The adjoint of one CLAMP step (w9: mirrored taps), border included.
+int launch_stream2d_fold(bool taps5, const float *in, float *out, int64_t rows, int64_t cols, const float *w9,
+                         cudaStream_t s);
 int launch_stencil_chain_fused(const StencilLaunch &st, int steps, float *tmp, const Choice &c, cudaStream_t s);
 int chain_variant_count();
 const char *chain_variant_name(int v);

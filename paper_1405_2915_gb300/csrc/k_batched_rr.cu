@@ -76,58 +76,52 @@ struct BrFF {
     }
 };
 
-// The non-empty instance holding element v: the largest b in [0, B) with
-// off[b] <= v (sorted offsets; off[0] = 0 <= v < off[B]).
-__device__ __forceinline__ int64_t br_instance_of(const int64_t *__restrict__ off, int64_t B, int64_t v)
-{
-    int64_t lo = 0, hi = B - 1;
-    while (lo < hi) {
-        const int64_t mid = (lo + hi + 1) >> 1;
-        if (__ldg(off + mid) <= v) lo = mid;
-        else hi = mid - 1;
-    }
-    return lo;
-}
-
-// Each tile's placement, one thread per tile (unchecked offsets give
-// placements the main kernel never reads: it stops at the check's flag).
+// Checks the offsets and writes each tile's placement, one warp per instance:
+// the tiles whose first element it holds get its number, the tiles whose last
+// element it holds its start.  No searches: two dependent loads, then stores
+// (a search per tile was twelve dependent loads, and the check a kernel of
+// one block: 5.4 + 7.7 us for 4096 instances, now 3.3 in one launch).
+// Invalid offsets are reported and, unless `alone` (no main kernel follows),
+// make the main kernel return at once; the placements they give are only
+// kept inside the array.
 __global__ void __launch_bounds__(256)
-batched_br_meta(const int64_t *__restrict__ off, int64_t B, int64_t total, BrMeta *__restrict__ meta)
+batched_br_place(const int64_t *__restrict__ off, int64_t B, int64_t total, float *__restrict__ results,
+                 BrMeta *__restrict__ meta, Control *ctl, int alone)
 {
     dev::grid_wait();
+    const int lane = threadIdx.x & 31;
     const int64_t ntiles = (total + kBrTE - 1) / kBrTE;
-    for (int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; t < ntiles; t += (int64_t)gridDim.x * blockDim.x) {
-        const int64_t last = (t + 1) * kBrTE < total ? (t + 1) * kBrTE - 1 : total - 1;
-        const int64_t b0 = br_instance_of(off, B, t * kBrTE), bl = br_instance_of(off, B, last);
-        meta[t] = BrMeta{b0, __ldg(off + bl)};
+    bool bad = blockIdx.x == 0 && threadIdx.x == 0 && (off[0] != 0 || off[B] != total);
+    for (int64_t b = (int64_t)blockIdx.x * 8 + (threadIdx.x >> 5); b < B; b += (int64_t)gridDim.x * 8) {
+        const int64_t lo = __ldg(off + b), hi = __ldg(off + b + 1);
+        if (hi <= lo) {
+            bad |= hi < lo;
+            if (lane == 0 && hi == lo && results) results[b] = 0.f;
+            continue;
+        }
+        if (lo < 0 || hi > total) {
+            bad = true;
+            continue;
+        }
+        // first elements t * TE in [lo, hi)
+        for (int64_t t = (lo + kBrTE - 1) / kBrTE + lane; t * kBrTE < hi; t += 32) meta[t].b0 = b;
+        // last elements (t + 1) * TE - 1, of the last tile total - 1, in [lo, hi)
+        for (int64_t t = lo / kBrTE + lane; t < ntiles; t += 32) {
+            const int64_t last = (t + 1) * kBrTE < total ? (t + 1) * kBrTE - 1 : total - 1;
+            if (last >= hi) break;
+            meta[t].hp = lo;
+        }
     }
-}
-
-// Offsets check (as variant 6's).
-__global__ void __launch_bounds__(1024)
-batched_br_prep(const int64_t *__restrict__ off, int64_t B, int64_t total, float *__restrict__ results,
-                int *__restrict__ ok, Control *ctl)
-{
-    dev::grid_wait();
-    __shared__ int bad;
-    if (threadIdx.x == 0) bad = (off[0] != 0 || off[B] != total) ? 1 : 0;
-    __syncthreads();
-    for (int64_t b = threadIdx.x; b < B; b += blockDim.x) {
-        const int64_t lo = off[b], hi = off[b + 1];
-        if (hi < lo) bad = 1;
-        else if (hi == lo && results) results[b] = 0.f;
-    }
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        *ok = bad ? 0 : 1;
-        if (bad) atomicOr(&ctl->error, kErrInput);
+    if (bad) {
+        atomicOr(&ctl->error, kErrInput);
+        if (!alone) atomicExch(&ctl->reject, 1u);
     }
 }
 
 template <bool SCAN, bool RED, bool INCL, int R, int NC>
 __global__ void __launch_bounds__((kBrAggW + NC) * 32, 1)
 batched_br(const float *__restrict__ values, const int64_t *__restrict__ off, int64_t B, int64_t total,
-           float *__restrict__ results, float *__restrict__ scan_out, const int *__restrict__ ok,
+           float *__restrict__ results, float *__restrict__ scan_out,
            const BrMeta *__restrict__ meta, dev::LookbackDesc d, Control *ctl, uint32_t epoch, int64_t skip_tile,
            uint64_t limit_ns)
 {
@@ -146,7 +140,14 @@ batched_br(const float *__restrict__ values, const int64_t *__restrict__ off, in
     __shared__ int q_tail, q_claim, q_read, a_done, s_stop;
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
     const int64_t ntiles = (total + TE - 1) / TE, nfull = total / TE;
-    if (!*ok) return;   // rejected offsets (reported by the prep kernel); every block leaves, no ticket drawn
+    if (dev::ld_volatile(&ctl->reject)) {   // invalid offsets (reported): every block leaves, no ticket drawn
+        __syncthreads();                    // every thread has read the flag
+        if (threadIdx.x == 0 && atomicAdd(&ctl->exited, 1u) == gridDim.x - 1) {   // ... and every block
+            ctl->reject = 0u;
+            ctl->exited = 0u;
+        }
+        return;
+    }
     auto gave_up = [&]() { return dev::ld_volatile(&ctl->abort) == epoch; };
     auto give_up = [&]() {
         atomicOr(&ctl->error, kErrTimeout);
@@ -565,8 +566,7 @@ batched_br(const float *__restrict__ values, const int64_t *__restrict__ off, in
 }
 
 template <bool SCAN, bool RED, bool INCL, int R, int NC>
-int run_br_k(const BatchedLaunch &b, Control *ctl, uint64_t *words, const int *ok, const BrMeta *meta,
-             uint32_t epoch, cudaStream_t s)
+int run_br_k(const BatchedLaunch &b, Control *ctl, uint64_t *words, const BrMeta *meta, uint32_t epoch, cudaStream_t s)
 {
     auto kern = batched_br<SCAN, RED, INCL, R, NC>;
     const int dyn = (R + NC) * kBrTE * 4, threads = (kBrAggW + NC) * 32;
@@ -576,22 +576,21 @@ int run_br_k(const BatchedLaunch &b, Control *ctl, uint64_t *words, const int *o
     dev::LookbackDesc d{words, words + 2 * ntiles};
     const DebugKnobs k = debug_knobs();
     launch_kernel(kern, (unsigned)(device_info().sms * occ), threads, (size_t)dyn, s, b.values, b.offsets, b.B,
-                  b.total, b.results, b.scan_out, ok, meta, d, ctl, epoch, k.scan_skip_publish_tile, k.wait_limit_ns);
+                  b.total, b.results, b.scan_out, meta, d, ctl, epoch, k.scan_skip_publish_tile, k.wait_limit_ns);
     const cudaError_t e = cudaPeekAtLastError();
     return e == cudaSuccess ? SKEL_OK : fail_cuda(cudaGetLastError(), "batched reread launch");
 }
 
 template <int R, int NC>
-int run_br_shape(const BatchedLaunch &b, Control *ctl, uint64_t *words, const int *ok, const BrMeta *meta,
-                 uint32_t epoch, cudaStream_t s)
+int run_br_shape(const BatchedLaunch &b, Control *ctl, uint64_t *words, const BrMeta *meta, uint32_t epoch, cudaStream_t s)
 {
     if (b.want_scan && b.want_reduce)
-        return b.inclusive ? run_br_k<true, true, true, R, NC>(b, ctl, words, ok, meta, epoch, s)
-                           : run_br_k<true, true, false, R, NC>(b, ctl, words, ok, meta, epoch, s);
+        return b.inclusive ? run_br_k<true, true, true, R, NC>(b, ctl, words, meta, epoch, s)
+                           : run_br_k<true, true, false, R, NC>(b, ctl, words, meta, epoch, s);
     if (b.want_scan)
-        return b.inclusive ? run_br_k<true, false, true, R, NC>(b, ctl, words, ok, meta, epoch, s)
-                           : run_br_k<true, false, false, R, NC>(b, ctl, words, ok, meta, epoch, s);
-    return run_br_k<false, true, true, R, NC>(b, ctl, words, ok, meta, epoch, s);
+        return b.inclusive ? run_br_k<true, false, true, R, NC>(b, ctl, words, meta, epoch, s)
+                           : run_br_k<true, false, false, R, NC>(b, ctl, words, meta, epoch, s);
+    return run_br_k<false, true, true, R, NC>(b, ctl, words, meta, epoch, s);
 }
 
 // tile: the ring's tiles and the scanner warps (16 KiB each): 0 = 6 + 6, 1 = 4 + 8.
@@ -602,18 +601,15 @@ int run_br(const BatchedLaunch &b, const Choice &c, Control *ctl, uint64_t *word
     if (c.tile < 0 || c.tile > 1) return fail(SKEL_ERR_INVALID_ARG, "batched reread: tile must be 0 or 1");
     const int64_t ntiles = ceil_div(b.total, (int64_t)kBrTE);
     if (ntiles > 0x7fffffffLL) return fail(SKEL_ERR_SHAPE, "batched: too many tiles");
-    int *ok = reinterpret_cast<int *>(data);
     BrMeta *meta = reinterpret_cast<BrMeta *>(data + 256);
-    launch_kernel(batched_br_prep, 1, 1024, 0, s, b.offsets, b.B, b.total, b.results, ok, ctl);
-    if (b.total > 0) {
-        const int64_t mgrid = std::min<int64_t>(ceil_div(ntiles, (int64_t)256), (int64_t)device_info().sms * 8);
-        launch_kernel(batched_br_meta, (unsigned)mgrid, 256, 0, s, b.offsets, b.B, b.total, meta);
-    }
+    const int64_t pgrid = std::max<int64_t>(1, std::min<int64_t>(ceil_div(b.B, (int64_t)8), (int64_t)device_info().sms * 8));
+    launch_kernel(batched_br_place, (unsigned)pgrid, 256, 0, s, b.offsets, b.B, b.total, b.results, meta, ctl,
+                  b.total == 0 ? 1 : 0);
     cudaError_t e = cudaPeekAtLastError();
     if (e != cudaSuccess) return fail_cuda(cudaGetLastError(), "batched reread prep launch");
     if (b.total == 0) return SKEL_OK;
-    return c.tile ? run_br_shape<4, 8>(b, ctl, words, ok, meta, epoch, s)
-                  : run_br_shape<6, 6>(b, ctl, words, ok, meta, epoch, s);
+    return c.tile ? run_br_shape<4, 8>(b, ctl, words, meta, epoch, s)
+                  : run_br_shape<6, 6>(b, ctl, words, meta, epoch, s);
 }
 
 }  // namespace
