@@ -29,8 +29,9 @@
 // the same boundary for ZERO and PERIODIC.  For CLAMP, taps that the forward
 // pass clamped onto an edge element fold their weight back onto that edge:
 // only the first and last row/column (1D: the two end elements) receive such
-// folded terms, so the interior runs the mirrored stencil and a fix-up kernel
-// rewrites the border with the exact folded sums.
+// folded terms: the row stream adds them as the edge rows and columns pass;
+// the other variants run the mirrored stencil and a fix-up kernel that
+// rewrites the border with the exact folded sums (4 us more).
 #include <cuda.h>
 
 #include <mutex>
@@ -549,7 +550,11 @@ const char *stencil_variant_name(int ndim, int v)
     if (ndim == 1) return v >= 0 && v < 3 ? n1[v] : "?";
     return v >= 0 && v < 4 ? n2[v] : "?";
 }
-Choice stencil_default(int ndim) { return ndim == 1 ? Choice{1, 256, 8, 0} : Choice{1, 256, 0, 0}; }
+// 2D: the row stream beats the shared-memory tile at every size (9-point,
+// forward: 512^2 2.6 us against 3.8, 2048^2 6.9 against 10.3, 8192^2 93
+// against 125); the TMA tile is ahead of it from 4096^2 (25.2; 8192^2 81),
+// which the table takes.
+Choice stencil_default(int ndim) { return ndim == 1 ? Choice{1, 256, 8, 0} : Choice{0, 256, 0, 0}; }
 
 int launch_stencil(const StencilLaunch &st, const Choice &c, cudaStream_t s)
 {
@@ -562,6 +567,8 @@ int launch_stencil(const StencilLaunch &st, const Choice &c, cudaStream_t s)
         for (int k = 0; k < 9; ++k) w.w[k] = st.w[k];
         for (int k = 0; k < 9; ++k) wf.w[k] = st.transpose ? st.w[8 - k] : st.w[k];
         if (st.taps5) { wf.w[0] = wf.w[2] = wf.w[6] = wf.w[8] = 0.f; w.w[0] = w.w[2] = w.w[6] = w.w[8] = 0.f; }
+        if (c.variant == 0 && st.transpose && st.boundary == SKEL_CLAMP)   // border included
+            return launch_stream2d_fold(st.taps5, st.in, st.out, st.rows, st.cols, wf.w, s);
         int rc = st.taps5 ? run2d<true>(st, c, st.in, st.out, b, wf, s) : run2d<false>(st, c, st.in, st.out, b, wf, s);
         if (rc || !st.transpose || st.boundary != SKEL_CLAMP) return rc;
         const int64_t nb = st.rows * st.cols;   // upper bound of border cells

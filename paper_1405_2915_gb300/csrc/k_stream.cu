@@ -60,9 +60,12 @@ struct StreamGeom {
 };
 
 // VEC: rows start on 16-byte boundaries (in, out aligned, cols % 4 == 0).
+// FOLD (one step, ZERO): the adjoint of a CLAMP stencil: w are the mirrored
+// taps, and what a cell beside the grid would receive goes to the edge cell it
+// stands for (taps that the forward pass clamped onto that cell).
 // H: output rows per segment; strips: strips per row of the grid; nwork:
 // strips * segments.
-template <bool TAPS5, int K, bool VEC>
+template <bool TAPS5, int K, bool VEC, bool FOLD>
 __global__ void __launch_bounds__(32 * kStreamWarps)
 st2_stream(const float *__restrict__ in, float *__restrict__ out, int64_t rows, int64_t cols, int b, W9 w, int H,
            int64_t strips, int64_t nwork)
@@ -173,13 +176,39 @@ st2_stream(const float *__restrict__ in, float *__restrict__ out, int64_t rows, 
                     if (!TAPS5) o = fmaf(w.w[6], e[j], o);
                     o = fmaf(w.w[7], e[j + 1], o);
                     if (!TAPS5) o = fmaf(w.w[8], e[j + 2], o);
-                    x[j] = o;
+                    x[j] = o;   // (e still holds the row)
                     P2[s][j] = fmaf(w.w[5], e[j + 2], fmaf(w.w[4], e[j + 1], fmaf(w.w[3], e[j], P1[s][j])));
                     float n = 0.f;
                     if (!TAPS5) n = fmaf(w.w[0], e[j], n);
                     n = fmaf(w.w[1], e[j + 1], n);
                     if (!TAPS5) n = fmaf(w.w[2], e[j + 2], n);
                     P1[s][j] = n;
+                }
+                if (FOLD && (ROWE || COLE)) {
+                    // the first row also receives what the row above the grid would, the last row what the row below would
+                    const bool up = ROWE && top && i == 0, down = ROWE && bottom && i == nin - 1;
+#pragma unroll
+                    for (int j = 0; j < C; ++j) {
+                        if (up) P2[0][j] = fmaf(w.w[8], e[j + 2], fmaf(w.w[7], e[j + 1], fmaf(w.w[6], e[j], P2[0][j])));
+                        if (down) P2[0][j] = fmaf(w.w[2], e[j + 2], fmaf(w.w[1], e[j + 1], fmaf(w.w[0], e[j], P2[0][j])));
+                        if (!COLE) continue;
+                        // likewise the columns beside the grid: one tap per row of the first, of the last column
+                        const float v = e[j + 1];
+                        if (lead && j == 0) {
+                            x[j] = fmaf(w.w[8], v, x[j]);
+                            P2[0][j] = fmaf(w.w[5], v, P2[0][j]);
+                            P1[0][j] = fmaf(w.w[2], v, P1[0][j]);
+                            if (up) P2[0][j] = fmaf(w.w[8], v, P2[0][j]);
+                            if (down) P2[0][j] = fmaf(w.w[2], v, P2[0][j]);
+                        }
+                        if (trail && j == nv - 1) {
+                            x[j] = fmaf(w.w[6], v, x[j]);
+                            P2[0][j] = fmaf(w.w[3], v, P2[0][j]);
+                            P1[0][j] = fmaf(w.w[0], v, P1[0][j]);
+                            if (up) P2[0][j] = fmaf(w.w[6], v, P2[0][j]);
+                            if (down) P2[0][j] = fmaf(w.w[0], v, P2[0][j]);
+                        }
+                    }
                 }
             }
             if (i >= ifirst) store(x);
@@ -207,11 +236,11 @@ st2_stream(const float *__restrict__ in, float *__restrict__ out, int64_t rows, 
 // K = 5: 2K, K rows 18.8, 14.6 us).
 constexpr int kStreamFill = 16;
 
-template <bool TAPS5, int K, bool VEC>
+template <bool TAPS5, int K, bool VEC, bool FOLD = false>
 int run_stream(const float *in, float *out, int64_t rows, int64_t cols, int b, const W9 &w, cudaStream_t s)
 {
     using G = StreamGeom<K>;
-    auto kern = st2_stream<TAPS5, K, VEC>;
+    auto kern = st2_stream<TAPS5, K, VEC, FOLD>;
     const int occ = kernel_occupancy(kern, 32 * kStreamWarps, G::smem_bytes);
     if (occ < 1) return fail(SKEL_ERR_UNSUPPORTED, "mapoverlap stream: kernel does not fit an SM");
     const int64_t strips = ceil_div(cols, (int64_t)G::W);
@@ -254,7 +283,23 @@ int run_stream_taps(int k, const float *in, float *out, int64_t rows, int64_t co
     }
 }
 
+template <bool TAPS5>
+int run_stream_fold(const float *in, float *out, int64_t rows, int64_t cols, const W9 &w, cudaStream_t s)
+{
+    return cols % 4 == 0 && aligned16(in) && aligned16(out)
+               ? run_stream<TAPS5, 1, true, true>(in, out, rows, cols, SKEL_ZERO, w, s)
+               : run_stream<TAPS5, 1, false, true>(in, out, rows, cols, SKEL_ZERO, w, s);
+}
+
 }  // namespace
+
+int launch_stream2d_fold(bool taps5, const float *in, float *out, int64_t rows, int64_t cols, const float *w9,
+                         cudaStream_t s)
+{
+    W9 w;
+    for (int q = 0; q < 9; ++q) w.w[q] = w9[q];
+    return taps5 ? run_stream_fold<true>(in, out, rows, cols, w, s) : run_stream_fold<false>(in, out, rows, cols, w, s);
+}
 
 int launch_stream2d(bool taps5, int k, const float *in, float *out, int64_t rows, int64_t cols, int b, const float *w9,
                     cudaStream_t s)
