@@ -149,11 +149,49 @@ struct ScratchBlock {
     size_t data_cap = 0;    // bytes
     uint32_t epoch = 0;
     Allocator alloc{};
+    bool captured = false;  // a graph captured on the stream may hold its address
 };
+struct RetiredBlock {
+    int dev;
+    cudaStream_t stream;
+    void *base;
+    Allocator alloc;
+};
+std::vector<RetiredBlock> g_retired;   // replaced blocks that a graph may hold; freed by skel_release_cached
 std::mutex g_scr_mu;
 std::map<std::pair<int, cudaStream_t>, ScratchBlock> g_scratch;
 
 size_t round256(size_t b) { return (b + 255) & ~(size_t)255; }
+
+bool is_capturing(cudaStream_t stream)
+{
+    cudaStreamCaptureStatus st = cudaStreamCaptureStatusNone;
+    if (cudaStreamIsCapturing(stream, &st) != cudaSuccess) {
+        cudaGetLastError();   // the legacy stream while another stream captures
+        return false;
+    }
+    return st == cudaStreamCaptureStatusActive;
+}
+
+// Zeroed memory for a block that `stream` needs while it is being captured:
+// made on a stream of its own, so that it is neither a node of the graph nor
+// bound to its lifetime.
+void *alloc_beside_capture(size_t bytes)
+{
+    cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;
+    if (cudaThreadExchangeStreamCaptureMode(&mode) != cudaSuccess) return nullptr;
+    void *p = nullptr;
+    cudaStream_t side;
+    if (cudaStreamCreateWithFlags(&side, cudaStreamNonBlocking) == cudaSuccess) {
+        p = dev_alloc(Allocator{nullptr, nullptr, nullptr}, bytes, side);
+        if (p && cudaMemsetAsync(p, 0, bytes, side) != cudaSuccess) p = nullptr;
+        if (cudaStreamSynchronize(side) != cudaSuccess) p = nullptr;
+        cudaStreamDestroy(side);
+    }
+    cudaGetLastError();
+    cudaThreadExchangeStreamCaptureMode(&mode);
+    return p;
+}
 }  // namespace
 
 int get_scratch(cudaStream_t stream, size_t data_bytes, size_t word_count, Scratch *out)
@@ -163,6 +201,9 @@ int get_scratch(cudaStream_t stream, size_t data_bytes, size_t word_count, Scrat
     std::lock_guard<std::mutex> lk(g_scr_mu);
     ScratchBlock &b = g_scratch[{dev, stream}];
     const bool grow = !b.base || data_bytes > b.data_cap || word_count > b.word_cap;
+    // a block whose address a captured graph holds is kept when a larger one
+    // replaces it: a replay still uses it
+    const bool capturing = is_capturing(stream);
     if (grow) {
         size_t wc = std::max(word_count, b.word_cap);
         size_t dc = std::max(data_bytes, b.data_cap);
@@ -173,10 +214,12 @@ int get_scratch(cudaStream_t stream, size_t data_bytes, size_t word_count, Scrat
         }
         wc = std::max<size_t>(round256(wc * 8) / 8, 32);
         dc = std::max<size_t>(round256(dc), 256);
-        if (b.base) dev_free(b.alloc, b.base, stream);
-        b.alloc = current_allocator();
+        if (b.base && (b.captured || capturing)) g_retired.push_back(RetiredBlock{dev, stream, b.base, b.alloc});
+        else if (b.base) dev_free(b.alloc, b.base, stream);
+        b.captured = false;
+        b.alloc = capturing ? Allocator{nullptr, nullptr, nullptr} : current_allocator();
         const size_t total = sizeof(Control) + wc * 8 + dc;
-        b.base = dev_alloc(b.alloc, total, stream);
+        b.base = capturing ? alloc_beside_capture(total) : dev_alloc(b.alloc, total, stream);
         if (!b.base) {
             b = ScratchBlock{};
             return fail(SKEL_ERR_OOM, "scratch allocation failed");
@@ -184,9 +227,12 @@ int get_scratch(cudaStream_t stream, size_t data_bytes, size_t word_count, Scrat
         b.word_cap = wc;
         b.data_cap = dc;
         b.epoch = 0;
-        cudaError_t e = cudaMemsetAsync(b.base, 0, total, stream);
-        if (e != cudaSuccess) return fail_cuda(e, "scratch clear");
+        if (!capturing) {
+            cudaError_t e = cudaMemsetAsync(b.base, 0, total, stream);
+            if (e != cudaSuccess) return fail_cuda(e, "scratch clear");
+        }
     }
+    b.captured |= capturing;
     unsigned char *base = static_cast<unsigned char *>(b.base);
     out->ctl = reinterpret_cast<Control *>(base);
     out->words = reinterpret_cast<uint64_t *>(base + sizeof(Control));
@@ -300,6 +346,13 @@ int release_scratch()
         dev_free(kv.second.second, kv.second.first, kv.first.second);
     }
     cudaSetDevice(cur);
+    for (const RetiredBlock &r : g_retired) {
+        cudaSetDevice(r.dev);
+        cudaStreamSynchronize(r.stream);
+        dev_free(r.alloc, r.base, r.stream);
+    }
+    cudaSetDevice(cur);
+    g_retired.clear();
     g_scratch.clear();
     g_slots.clear();
     {

@@ -69,3 +69,37 @@ def test_two_streams_share_a_container():
         sk.skel_map("add", [cs[k % 2], cs[2]], cs[(k + 1) % 2], stream=streams[k % 2])
     torch.cuda.synchronize()
     assert np.array_equal(a.cpu().numpy(), np.full(N, 200, np.float32))
+
+
+def test_capture_on_a_stream_without_scratch_and_growth_afterwards():
+    """The first call on a stream happens inside a capture: the graph's
+    scratch is neither its own node nor freed when a later call on the stream
+    needs more."""
+    import torch
+    sk = skel()
+    s = torch.cuda.Stream()
+    x = torch.rand(600, 700, device="cuda") * 2 - 1
+    r = torch.zeros(2, device="cuda")
+    cx, cflat, ca, cb = wrap(x), wrap(x.reshape(-1)), wrap(r[0:1]), wrap(r[1:2])
+    torch.cuda.synchronize()
+    g = torch.cuda.CUDAGraph()
+    sk.skel_force_variant("compose", 2)
+    try:
+        with torch.cuda.graph(g, stream=s):
+            sk.skel_compose_map_stencil_sumsq("tanh", "stencil9", cx, result_dev=ca, host=False)
+            sk.skel_reduce("max", cflat, cb, host=False)
+        want = sk.skel_compose_map_stencil_sumsq("tanh", "stencil9", cx)
+        for k in range(3):
+            r.zero_()
+            torch.cuda.synchronize()
+            g.replay()
+            torch.cuda.synchronize()
+            assert float(r[0]) == float(want) and float(r[1]) == float(x.max())
+            big = torch.rand(1 << (16 + 3 * k), device="cuda")   # more scratch on the same stream
+            out = torch.empty_like(big)
+            with torch.cuda.stream(s):
+                sk.skel_scan("add", True, wrap(big), wrap(out))
+                sk.skel_reduce("add", wrap(big), cb, host=False)
+            s.synchronize()
+    finally:
+        sk.skel_force_variant("compose", -1)
