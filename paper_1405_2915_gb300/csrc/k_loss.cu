@@ -18,20 +18,22 @@
 // local sums, a warp scan, and the sum of the other warps' totals.
 // The forward needs one block barrier per row, the backward two (the scan's
 // totals and the second stencil's edges travel with the first stencil's).
-// Rows come through a ring in shared memory filled by cp.async: each row as
-// C / 4 planes (plane p holds the p-th group of four columns of every thread,
-// so 16-byte reads are free of bank conflicts); a row's slot also carries the
-// finished row back out, so that global stores are contiguous per warp.
+// Rows come through a ring in shared memory, three of them in flight, and a
+// row's slot also carries the finished row back out.  Aligned rows of a
+// multiple of 16 columns travel as TMA boxes, others by cp.async into C / 4
+// planes (plane p holds the p-th group of four columns of every thread, so
+// 16-byte reads are free of bank conflicts) and out by contiguous stores.
 //
-// What bounds it (8192 x 8192): the forward takes 180 us, the backward 235,
-// against 79 us each for their HBM traffic (which ncu shows at 1.0 of the
-// algorithmic bytes): instruction issue at 50 % of its peak with 16 warps per
-// SM whose barriers keep them in the same phase (51 and 69 instructions per
-// 32 points: two MUFUs and about 15 others of tanhf, 9 FMAs per stencil, 5 to
-// 6 per scan).  The forward computes the next row's tanh beside this row's
-// sums for that reason.  As fifteen separate calls the loss and its gradient
-// took 927 us, here 410.  512 threads of 16 columns: with 1024 of 8 the
-// scans' shuffles and the edges weigh twice as much.
+// What bounds it (8192 x 8192): the forward takes 136 us, the backward 176
+// (180 and 235 with cp.async), against 79 us each for their HBM traffic
+// (which ncu shows at 1.0 of the algorithmic bytes): instruction issue, which
+// alone takes 80 and 107 us, with 16 warps per SM whose barriers keep them in
+// the same phase (about 50 and 68 instructions per 32 points: two MUFUs and
+// about 15 others of tanhf, 9 FMAs per stencil, 5 to 6 per scan).  The forward
+// computes the next row's tanh beside this row's sums for that reason.  As
+// fifteen separate calls the loss and its gradient took 927 us, here 315.  512
+// threads of 16 columns: with 1024 of 8 the scans' shuffles and the edges
+// weigh twice as much.
 //
 // Sums run per thread with their rounding errors kept, then in float64 over
 // threads and blocks; the last block to finish adds the blocks' partial sums
@@ -43,10 +45,15 @@
 namespace skel {
 namespace {
 
-constexpr int kFwdC = 16, kBwdC = 16;         // columns per thread (forward with 8: 203 us for 180)
+constexpr int kFwdC = 16, kBwdC = 16;         // columns per thread (forward with 8: 203 us for 180, with cp.async)
 constexpr int kLMaxCols = 8192;
 constexpr int kLWarps = 32;                   // most warps of a block
 constexpr int kFwdRing = 4, kBwdRing = 6;     // rows in shared memory; 3 of them in flight
+
+// How rows travel: 4-byte copies, 16-byte copies (aligned rows), or TMA boxes
+// of one warp's columns (aligned rows of a multiple of 16 columns).
+enum { kCopy4, kCopy16, kTma };
+constexpr int kSwizzleAlign = 1024;           // TMA: alignment of the ring
 
 // Floats of one ring row of `threads` threads with C columns each: C / 4
 // planes of 4 floats per thread, each plane 32 / (C / 4) floats longer so that
@@ -118,7 +125,16 @@ __device__ __forceinline__ double warp_sum(double v)
 
 // The part of a thread's work both directions share: its columns, the ring,
 // the edges of the row.
-template <bool VEC, int C>
+//
+// With TMA the row's layout is the grid's own: 64 bytes per thread, the four
+// 16-byte groups swizzled by the lane (SWIZZLE_64B) so that each group's reads
+// meet every bank once.  A warp loads, reads, rewrites and stores its own 2 KB
+// only, each load completing on the warp's own mbarrier of the slot, so the
+// copies need no block barrier and take none of the load/store unit's issue:
+// the plane copies of 16 bytes per lane (32 KB per row in 64 instructions,
+// queued ahead of the shuffles and edge reads behind the barrier) cost the
+// forward 57 of its 183 us and the backward 67 of 241 (timed without them).
+template <int MODE, int C, int R>
 struct RowStream {
     static constexpr int NP = C / 4;   // planes
     int nthr, lane, warp, nwarps, nv, pf;
@@ -127,10 +143,16 @@ struct RowStream {
     float *ring;
     uint32_t ring_s;
     const float *next;            // row of the next copy, at this thread's first element
-    int nrows, ncopied, ringlen;
+    int nrows, ncopied;
+    // TMA
+    const CUtensorMap *tin, *tout;
+    Control *ctl;
+    uint32_t bar_s;               // the warp's R mbarriers
+    int q0i;                      // first row of the block
+    bool ok;                      // no wait has run out
 
     __device__ __forceinline__ RowStream(const float *in, int64_t rows_, int64_t cols_, int64_t q0, int nin, float *ring_,
-                                         int ringlen_)
+                                         const CUtensorMap *tin_, const CUtensorMap *tout_, Control *ctl_)
     {
         nthr = blockDim.x;
         lane = threadIdx.x & 31;
@@ -145,12 +167,27 @@ struct RowStream {
         lead = threadIdx.x == 0;
         trail = n > 0 && n <= C;
         cedge = warp == 0 || (warp + 1) * 32 * C >= cols;
-        ring = ring_;
-        ring_s = (uint32_t)__cvta_generic_to_shared(ring_);
+        ring = MODE == kTma ? ring_ + (0u - (uint32_t)__cvta_generic_to_shared(ring_)) % kSwizzleAlign / 4 : ring_;
+        ring_s = (uint32_t)__cvta_generic_to_shared(ring);
         next = in + q0 * cols;
         nrows = nin;
         ncopied = 0;
-        ringlen = ringlen_;
+        tin = tin_;
+        tout = tout_;
+        ctl = ctl_;
+        q0i = (int)q0;
+        ok = true;
+        if constexpr (MODE == kTma) {
+            bar_s = ring_s + (uint32_t)(R * nthr * C) * 4u + (uint32_t)(warp * R) * 8u;
+            if (lane == 0) {
+#pragma unroll
+                for (int k = 0; k < R; ++k)
+                    asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" :: "r"(bar_s + 8u * k) : "memory");
+                asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+                asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+            }
+            __syncwarp();
+        }
     }
     // zeroes the columns past the grid (only the warps that hold some)
     __device__ __forceinline__ void mask(float (&v)[C]) const
@@ -160,13 +197,39 @@ struct RowStream {
             for (int j = 0; j < C; ++j) v[j] = j < nv ? v[j] : 0.f;
         }
     }
-    __device__ __forceinline__ float *slot(int i) const { return ring + (i % ringlen) * NP * pf; }
-    // starts the copy of the next row, if there is one
+    __device__ __forceinline__ float *slot(int i) const { return ring + (i % R) * NP * pf; }
+    // TMA: the warp's part of slot i, and this thread's p-th 16-byte group in it
+    __device__ __forceinline__ uint32_t tma_slot(int i) const
+    {
+        return ring_s + (uint32_t)((i % R) * nthr + warp * 32) * (C * 4);
+    }
+    __device__ __forceinline__ float *tma_group(int i, int p) const
+    {
+        return ring + ((i % R) * nthr + (int)threadIdx.x) * C + 4 * (p ^ (lane >> 1 & 3));
+    }
+    // Starts the copy of the next row, if there is one.  TMA: the store out of
+    // its slot, at most PENDING stores back, must have left shared memory.
+    template <int PENDING>
     __device__ __forceinline__ void copy_next()
     {
+        if constexpr (MODE == kTma) {
+            if (ncopied < nrows && ok) {
+                if (lane == 0) {
+                    const uint32_t bar = bar_s + 8u * (uint32_t)(ncopied % R);
+                    asm volatile("cp.async.bulk.wait_group.read %0;" :: "n"(PENDING) : "memory");
+                    asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" :: "r"(bar), "r"(32 * C * 4) : "memory");
+                    asm volatile("cp.async.bulk.tensor.3d.shared::cluster.global.tile.mbarrier::complete_tx::bytes"
+                                 " [%0], [%1, {%2, %3, %4}], [%5];"
+                                 :: "r"(tma_slot(ncopied)), "l"(tin), "r"(0), "r"(warp * 32), "r"(q0i + ncopied), "r"(bar)
+                                 : "memory");
+                }
+                ++ncopied;
+            }
+            return;
+        }
         if (ncopied < nrows) {
-            const uint32_t d = ring_s + (uint32_t)((ncopied % ringlen) * NP * pf) * 4u;
-            if (VEC) {
+            const uint32_t d = ring_s + (uint32_t)((ncopied % R) * NP * pf) * 4u;
+            if (MODE == kCopy16) {
 #pragma unroll
                 for (int m = 0; m < NP; ++m) {  // group q of four columns: plane q % NP, thread q / NP
                     const int q = m * nthr + threadIdx.x;
@@ -184,27 +247,64 @@ struct RowStream {
         }
         dev::cp_commit();
     }
+    // this thread's copies but the last N have landed (not with TMA)
+    template <int N>
+    __device__ __forceinline__ void landed() const
+    {
+        if constexpr (MODE != kTma) dev::cp_wait<N>();
+    }
+    // TMA: row i of the warp has landed.  After a bounded number of tries the
+    // error is recorded and the block goes on without copies or waits.
+    __device__ __forceinline__ bool await_once(int i) const
+    {
+        uint32_t done = 0;
+        for (uint32_t it = 0; it < (1u << 22) && !done; ++it)
+            asm volatile("{ .reg .pred p; mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2; selp.u32 %0, 1, 0, p; }"
+                         : "=r"(done) : "r"(bar_s + 8u * (uint32_t)(i % R)), "r"((uint32_t)(i / R & 1)) : "memory");
+        return __all_sync(0xffffffffu, done != 0);
+    }
+    __device__ __forceinline__ void await(int i)
+    {
+        if constexpr (MODE == kTma) {
+            if (ok && !await_once(i)) {
+                ok = false;
+                if (lane == 0) atomicOr(&ctl->error, kErrTimeout);
+            }
+        }
+    }
     __device__ __forceinline__ void read(int i, float (&v)[C]) const
     {
         const float *s = slot(i) + 4 * threadIdx.x;
 #pragma unroll
         for (int p = 0; p < NP; ++p) {
-            const float4 q = *reinterpret_cast<const float4 *>(s + p * pf);
+            const float4 q = *reinterpret_cast<const float4 *>(MODE == kTma ? tma_group(i, p) : s + p * pf);
             v[4 * p] = q.x; v[4 * p + 1] = q.y; v[4 * p + 2] = q.z; v[4 * p + 3] = q.w;
         }
     }
     // Writes v into the slot of row i (the warp's own part of it) and from
-    // there to the row `dst` of a grid.  The warp's lanes have read the slot.
-    __device__ __forceinline__ void write(int i, const float (&v)[C], float *dst) const
+    // there to row r of the grid out.  The warp's lanes have read the slot.
+    __device__ __forceinline__ void write(int i, const float (&v)[C], float *out, int64_t r) const
     {
-        float *s = slot(i);
+        if constexpr (MODE == kTma) {
+            __syncwarp();
+#pragma unroll
+            for (int p = 0; p < NP; ++p)
+                *reinterpret_cast<float4 *>(tma_group(i, p)) = make_float4(v[4 * p], v[4 * p + 1], v[4 * p + 2], v[4 * p + 3]);
+            asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+            __syncwarp();
+            if (lane == 0)
+                asm volatile("cp.async.bulk.tensor.3d.global.shared::cta.tile.bulk_group [%0, {%1, %2, %3}], [%4];"
+                             :: "l"(tout), "r"(0), "r"(warp * 32), "r"((int)r), "r"(tma_slot(i)) : "memory");
+            return;
+        }
+        float *s = slot(i), *dst = out + r * cols;
         __syncwarp();
 #pragma unroll
         for (int p = 0; p < NP; ++p)
             *reinterpret_cast<float4 *>(s + p * pf + 4 * threadIdx.x) =
                 make_float4(v[4 * p], v[4 * p + 1], v[4 * p + 2], v[4 * p + 3]);
         __syncwarp();
-        if (VEC) {
+        if (MODE == kCopy16) {
 #pragma unroll
             for (int m = 0; m < NP; ++m) {
                 const int q = warp * 32 * NP + 32 * m + lane;
@@ -218,6 +318,24 @@ struct RowStream {
                 const int e = warp * 32 * C + 32 * m + lane;
                 if (e < cols) dst[e] = s[(e / 4 % NP) * pf + (e / C) * 4 + e % 4];
             }
+        }
+    }
+    // TMA: closes the iteration's group of stores (which may be empty).
+    __device__ __forceinline__ void end_stores() const
+    {
+        if constexpr (MODE == kTma) {
+            if (lane == 0) asm volatile("cp.async.bulk.commit_group;" ::: "memory");
+        }
+    }
+    // Every copy of the thread has ended (three loads at most are in flight).
+    __device__ __forceinline__ void drain() const
+    {
+        if constexpr (MODE == kTma) {
+            if (!ok)
+                for (int k = ncopied > 3 ? ncopied - 3 : 0; k < ncopied; ++k) await_once(k);
+            if (lane == 0) asm volatile("cp.async.bulk.wait_group 0;" ::: "memory");
+        } else {
+            dev::cp_wait<0>();
         }
     }
 };
@@ -261,9 +379,9 @@ __device__ __forceinline__ float warp_offset(const Exchange &ex, int lane, int w
 }
 
 // ------------------------------------------------------------- forward --
-template <bool VEC>
+template <int MODE>
 __global__ void __launch_bounds__(kLMaxCols / kFwdC, 1)
-loss_fwd(const float *__restrict__ x, float *__restrict__ t_out, int64_t rows, int64_t cols, int b, W9 w, int H,
+loss_fwd(const __grid_constant__ CUtensorMap tin, const __grid_constant__ CUtensorMap tout, const float *__restrict__ x, float *__restrict__ t_out, int64_t rows, int64_t cols, int b, W9 w, int H,
          double2 *__restrict__ partials, float *__restrict__ L, Control *ctl)
 {
     dev::grid_wait();
@@ -276,15 +394,15 @@ loss_fwd(const float *__restrict__ x, float *__restrict__ t_out, int64_t rows, i
     const int64_t q0 = r0 > 0 ? r0 - 1 : 0;
     const bool top = r0 == 0, bottom = r1 == rows, clamp = b == SKEL_CLAMP;
     const int nin = (int)((bottom ? rows : r1 + 1) - q0);
-    RowStream<VEC, C> rs(x, rows, cols, q0, nin, dyn, kFwdRing);
+    RowStream<MODE, C, kFwdRing> rs(x, rows, cols, q0, nin, dyn, &tin, &tout, ctl);
     const int lane = rs.lane, warp = rs.warp;
     dev::Sum2 su, ss;
     float P1[C], P2[C];
 #pragma unroll
     for (int j = 0; j < C; ++j) P1[j] = P2[j] = 0.f;
 #pragma unroll
-    for (int k = 0; k < kFwdRing - 1; ++k) rs.copy_next();
-    dev::cp_wait<kFwdRing - 2>();
+    for (int k = 0; k < kFwdRing - 1; ++k) rs.template copy_next<1>();
+    rs.template landed<kFwdRing - 2>();
     __syncthreads();
 
     auto sum_sq = [&](float (&o)[C], dev::Sum2 &k) {   // the grid's columns only
@@ -296,6 +414,7 @@ loss_fwd(const float *__restrict__ x, float *__restrict__ t_out, int64_t rows, i
     };
     // t of row i (its copy has landed)
     auto load_t = [&](int i, float (&v)[C]) {
+        rs.await(i);
         rs.read(i, v);
 #pragma unroll
         for (int j = 0; j < C; ++j) v[j] = tanhf(v[j]);
@@ -308,7 +427,8 @@ loss_fwd(const float *__restrict__ x, float *__restrict__ t_out, int64_t rows, i
         Exchange &exi = ex[i & 1];
         const int64_t row = q0 + i;
         const bool own = row >= r0 && row < r1;
-        if (t_out && own) rs.write(i, v, t_out + row * cols);
+        if (t_out && own) rs.write(i, v, t_out, row);
+        rs.end_stores();
         float sc[C];
 #pragma unroll
         for (int j = 0; j < C; ++j) sc[j] = v[j];
@@ -318,9 +438,8 @@ loss_fwd(const float *__restrict__ x, float *__restrict__ t_out, int64_t rows, i
             exi.last[warp] = v[C - 1];
             exi.total[warp] = wi;
         }
-        dev::cp_wait<kFwdRing - 3>();   // row i + 1 has landed (its copies by every thread, after the barrier)
+        rs.template landed<kFwdRing - 3>();   // row i + 1 has landed (its copies by every thread, after the barrier)
         __syncthreads();
-        rs.copy_next();            // into the slot of row i - 1
         neighbours(v, exi, lane, warp, rs.nwarps, e);
         if (rs.cedge) {
             if (rs.lead) e[0] = clamp ? v[0] : 0.f;
@@ -340,6 +459,7 @@ loss_fwd(const float *__restrict__ x, float *__restrict__ t_out, int64_t rows, i
             for (int j = 0; j < C; ++j) sc[j] += base;
             sum_sq(sc, ss);
         }
+        rs.template copy_next<1>();   // into the slot of row i - 1; here, behind the row's other work: 136 us, right after the barrier 140
     }
     if (bottom) {                            // the row below the last one
         float o[C];
@@ -350,7 +470,7 @@ loss_fwd(const float *__restrict__ x, float *__restrict__ t_out, int64_t rows, i
         add_row(w, mid, e, P1, P2, o);
         sum_sq(o, su);
     }
-    dev::cp_wait<0>();
+    rs.drain();
     double a = warp_sum(su.value()), c = warp_sum(ss.value());
     if (lane == 0) red[warp] = make_double2(a, c);
     __syncthreads();
@@ -384,10 +504,10 @@ loss_fwd(const float *__restrict__ x, float *__restrict__ t_out, int64_t rows, i
 // Iteration i takes row q0 + i of t in, completes u of the row above it (the
 // upstream gradient gu = 2 g u of the second stencil), and completes gx of
 // the row above that.
-template <bool VEC>
+template <int MODE>
 __global__ void __launch_bounds__(kLMaxCols / kBwdC, 1)
-loss_bwd(const float *__restrict__ t, const float *__restrict__ g, float *__restrict__ gx, int64_t rows, int64_t cols,
-         int b, W9 w, int H)
+loss_bwd(const __grid_constant__ CUtensorMap tin, const __grid_constant__ CUtensorMap tout, const float *__restrict__ t, const float *__restrict__ g, float *__restrict__ gx, int64_t rows, int64_t cols,
+         int b, W9 w, int H, Control *ctl)
 {
     dev::grid_wait();
     constexpr int C = kBwdC;
@@ -397,7 +517,7 @@ loss_bwd(const float *__restrict__ t, const float *__restrict__ g, float *__rest
     const int64_t q0 = r0 > 2 ? r0 - 2 : 0;
     const bool clamp = b == SKEL_CLAMP;
     const int nin = (int)((r1 + 2 < rows ? r1 + 2 : rows) - q0), niter = (int)(r1 + 2 - q0);
-    RowStream<VEC, C> rs(t, rows, cols, q0, nin, dyn, kBwdRing);
+    RowStream<MODE, C, kBwdRing> rs(t, rows, cols, q0, nin, dyn, &tin, &tout, ctl);
     const int lane = rs.lane, warp = rs.warp;
     const float g2 = 2.f * __ldg(g), gc2 = 2.f * ((float)(1.0 / ((double)rows * (double)cols)) * __ldg(g));
     W9 wt;                                    // the mirrored taps of the adjoint
@@ -408,8 +528,8 @@ loss_bwd(const float *__restrict__ t, const float *__restrict__ g, float *__rest
     for (int j = 0; j < C; ++j) P1[j] = P2[j] = Q1[j] = Q2[j] = 0.f;
     float L1 = 0.f, L2 = 0.f, R1 = 0.f, R2 = 0.f;   // the columns beside the grid (below)
 #pragma unroll
-    for (int k = 0; k < 3; ++k) rs.copy_next();
-    dev::cp_wait<2>();
+    for (int k = 0; k < 3; ++k) rs.template copy_next<0>();
+    rs.template landed<2>();
     __syncthreads();
 
     for (int i = 0; i < niter; ++i) {
@@ -417,6 +537,7 @@ loss_bwd(const float *__restrict__ t, const float *__restrict__ g, float *__rest
         const bool out_row = row - 2 >= r0;   // (row - 2 < r1 by the loop's bound)
         // ---- phase 1: the arriving row, the scan of row - 2 ----
         float v[C];
+        if (i < nin) rs.await(i);
         rs.read(i < nin ? i : nin - 1, v);    // below the grid: the last row again (ZERO: 0)
         rs.mask(v);
         if (i >= nin && !clamp) {
@@ -435,7 +556,7 @@ loss_bwd(const float *__restrict__ t, const float *__restrict__ g, float *__rest
             ex[0].total[warp] = wi;
         }
         __syncthreads();
-        rs.copy_next();                       // into the slot of row i - 3
+        if (MODE != kTma) rs.template copy_next<0>();   // into the slot of row i - 3
         // ---- phase 2: u of row - 1, the reverse scan of row - 2 ----
         float e[C + 2];
         neighbours(v, ex[0], lane, warp, rs.nwarps, e);
@@ -474,8 +595,9 @@ loss_bwd(const float *__restrict__ t, const float *__restrict__ g, float *__rest
             ex[1].total[warp] = rwi;
         }
         if (lane == 31) ex[1].last[warp] = u[C - 1];
-        dev::cp_wait<2>();                         // row i + 1 has landed (visible after the barrier)
+        rs.template landed<2>();                   // row i + 1 has landed (visible after the barrier)
         __syncthreads();
+        if (MODE == kTma) rs.template copy_next<0>();   // here: the slot's store has had this row's two phases to end
         // ---- phase 3: the adjoint stencil of row - 2, gx of row - 2 ----
         neighbours(u, ex[1], lane, warp, rs.nwarps, e);    // 0 outside the grid
         // CLAMP: taps that the forward clamped onto the grid's edge.  The
@@ -514,10 +636,11 @@ loss_bwd(const float *__restrict__ t, const float *__restrict__ g, float *__rest
             rs.read(i - 2, y);
 #pragma unroll
             for (int j = 0; j < C; ++j) y[j] = (gt[j] + (sc[j] + base)) * fmaf(-y[j], y[j], 1.f);
-            rs.write(i - 2, y, gx + (row - 2) * cols);
+            rs.write(i - 2, y, gx, row - 2);
         }
+        rs.end_stores();
     }
-    dev::cp_wait<0>();
+    rs.drain();
 }
 
 // Threads of a block with C columns each: whole warps.
@@ -531,11 +654,31 @@ int rows_per_block(int64_t rows, int occ, int min_rows)
     return (int)(H < min_rows ? min_rows : H);
 }
 
-template <bool VEC>
-int run_fwd(const LossLaunch &l, cudaStream_t s)
+// A grid as rows of 16-column groups, in boxes of one warp's 32 groups.
+bool encode_rows(CUtensorMap *map, const float *p, int64_t rows, int64_t cols)
 {
-    const int nthr = threads_for(l.cols, kFwdC), smem = kFwdRing * row_floats<kFwdC>(nthr) * 4;
-    auto kern = loss_fwd<VEC>;
+    EncodeTiled enc = encode_tiled();
+    if (!enc) return false;
+    const cuuint64_t dims[3] = {16, (cuuint64_t)(cols / 16), (cuuint64_t)rows};
+    const cuuint64_t strides[2] = {64, (cuuint64_t)cols * 4};
+    const cuuint32_t box[3] = {16, 32, 1}, estr[3] = {1, 1, 1};
+    return enc(map, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 3, const_cast<float *>(p), dims, strides, box, estr,
+               CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_64B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
+               CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
+}
+
+// Dynamic shared memory: the ring, and with TMA its alignment and the warps' mbarriers.
+template <int MODE, int C, int R>
+int ring_bytes(int nthr)
+{
+    return MODE == kTma ? kSwizzleAlign + R * nthr * C * 4 + nthr / 32 * R * 8 : R * row_floats<C>(nthr) * 4;
+}
+
+template <int MODE>
+int run_fwd(const LossLaunch &l, const CUtensorMap &tin, const CUtensorMap &tout, cudaStream_t s)
+{
+    const int nthr = threads_for(l.cols, kFwdC), smem = ring_bytes<MODE, kFwdC, kFwdRing>(nthr);
+    auto kern = loss_fwd<MODE>;
     const int occ = kernel_occupancy(kern, nthr, smem);
     if (occ < 1) return fail(SKEL_ERR_UNSUPPORTED, "composed loss: kernel does not fit an SM");
     const int H = rows_per_block(l.rows, occ, 4);
@@ -545,24 +688,27 @@ int run_fwd(const LossLaunch &l, cudaStream_t s)
     if (rc) return rc;
     W9 w;
     for (int k = 0; k < 9; ++k) w.w[k] = l.w[k];
-    launch_kernel(kern, (unsigned)grid, nthr, (size_t)smem, s, l.x, l.t, l.rows, l.cols, l.boundary, w, H,
+    launch_kernel(kern, (unsigned)grid, nthr, (size_t)smem, s, tin, tout, l.x, l.t, l.rows, l.cols, l.boundary, w, H,
                   reinterpret_cast<double2 *>(scr.data), l.L, scr.ctl);
     cudaError_t e = cudaPeekAtLastError();
     return e == cudaSuccess ? SKEL_OK : fail_cuda(cudaGetLastError(), "composed loss launch");
 }
 
-template <bool VEC>
-int run_bwd(const LossLaunch &l, cudaStream_t s)
+template <int MODE>
+int run_bwd(const LossLaunch &l, const CUtensorMap &tin, const CUtensorMap &tout, cudaStream_t s)
 {
-    const int nthr = threads_for(l.cols, kBwdC), smem = kBwdRing * row_floats<kBwdC>(nthr) * 4;
-    auto kern = loss_bwd<VEC>;
+    const int nthr = threads_for(l.cols, kBwdC), smem = ring_bytes<MODE, kBwdC, kBwdRing>(nthr);
+    auto kern = loss_bwd<MODE>;
     const int occ = kernel_occupancy(kern, nthr, smem);
     if (occ < 1) return fail(SKEL_ERR_UNSUPPORTED, "composed loss: kernel does not fit an SM");
     const int H = rows_per_block(l.rows, occ, 4);
+    Scratch scr{};
+    int rc = get_scratch(s, 0, 0, &scr);
+    if (rc) return rc;
     W9 w;
     for (int k = 0; k < 9; ++k) w.w[k] = l.w[k];
-    launch_kernel(kern, (unsigned)ceil_div(l.rows, (int64_t)H), nthr, (size_t)smem, s, (const float *)l.t, l.g, l.gx, l.rows,
-                  l.cols, l.boundary, w, H);
+    launch_kernel(kern, (unsigned)ceil_div(l.rows, (int64_t)H), nthr, (size_t)smem, s, tin, tout, (const float *)l.t, l.g,
+                  l.gx, l.rows, l.cols, l.boundary, w, H, scr.ctl);
     cudaError_t e = cudaPeekAtLastError();
     return e == cudaSuccess ? SKEL_OK : fail_cuda(cudaGetLastError(), "composed loss adjoint launch");
 }
@@ -580,9 +726,15 @@ int loss_fused_check(int64_t rows, int64_t cols, int boundary)
 
 int launch_loss(const LossLaunch &l, cudaStream_t s)
 {
-    const bool vec = l.cols % 4 == 0 && aligned16(l.gx ? (const void *)l.gx : (const void *)l.x) && aligned16(l.t);
-    if (l.gx) return vec ? run_bwd<true>(l, s) : run_bwd<false>(l, s);
-    return vec ? run_fwd<true>(l, s) : run_fwd<false>(l, s);
+    const bool back = l.gx != nullptr;
+    const float *in = back ? l.t : l.x;
+    float *out = back ? l.gx : l.t;
+    const bool vec = l.cols % 4 == 0 && aligned16(in) && aligned16(out);
+    CUtensorMap tin{}, tout{};
+    if (vec && l.cols % 16 == 0 && encode_rows(&tin, in, l.rows, l.cols) && (!out || encode_rows(&tout, out, l.rows, l.cols)))
+        return back ? run_bwd<kTma>(l, tin, tout, s) : run_fwd<kTma>(l, tin, tout, s);
+    if (vec) return back ? run_bwd<kCopy16>(l, tin, tout, s) : run_fwd<kCopy16>(l, tin, tout, s);
+    return back ? run_bwd<kCopy4>(l, tin, tout, s) : run_fwd<kCopy4>(l, tin, tout, s);
 }
 
 }  // namespace skel

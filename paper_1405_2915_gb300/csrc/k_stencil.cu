@@ -422,26 +422,6 @@ __global__ void st1_fold_ends(const float *__restrict__ g, float *__restrict__ g
 }
 
 // ---------------------------------------------------------------- host --
-using EncodeTiled = CUresult (*)(CUtensorMap *, CUtensorMapDataType, cuuint32_t, void *, const cuuint64_t *,
-                                 const cuuint64_t *, const cuuint32_t *, const cuuint32_t *, CUtensorMapInterleave,
-                                 CUtensorMapSwizzle, CUtensorMapL2promotion, CUtensorMapFloatOOBfill);
-
-EncodeTiled encode_fn()
-{
-    static std::once_flag once;
-    static EncodeTiled fn = nullptr;
-    std::call_once(once, [] {
-        void *p = nullptr;
-        cudaDriverEntryPointQueryResult q;
-        if (cudaGetDriverEntryPointByVersion("cuTensorMapEncodeTiled", &p, 12000, cudaEnableDefault, &q) == cudaSuccess &&
-            q == cudaDriverEntryPointSuccess)
-            fn = reinterpret_cast<EncodeTiled>(p);
-        else
-            cudaGetLastError();
-    });
-    return fn;
-}
-
 int check_launch(const char *what)
 {
     cudaError_t e = cudaPeekAtLastError();
@@ -463,7 +443,7 @@ int run2d(const StencilLaunch &st, const Choice &c, const float *in, float *out,
         return check_launch("mapoverlap2d smem");
     }
     if (c.variant == 2) {
-        EncodeTiled enc = encode_fn();
+        EncodeTiled enc = encode_tiled();
         if (!enc) return fail(SKEL_ERR_UNSUPPORTED, "mapoverlap 2D: cuTensorMapEncodeTiled unavailable");
         if (rows > 0x7fffffff || cols > 0x7fffffff) return fail(SKEL_ERR_UNSUPPORTED, "TMA: grid too large");
         CUtensorMap map;
@@ -541,6 +521,22 @@ int run1d(const Choice &c, int r, const float *in, float *out, int64_t n, int b,
 }
 
 }  // namespace
+
+EncodeTiled encode_tiled()
+{
+    static std::once_flag once;
+    static EncodeTiled fn = nullptr;
+    std::call_once(once, [] {
+        void *p = nullptr;
+        cudaDriverEntryPointQueryResult q;
+        if (cudaGetDriverEntryPointByVersion("cuTensorMapEncodeTiled", &p, 12000, cudaEnableDefault, &q) == cudaSuccess &&
+            q == cudaDriverEntryPointSuccess)
+            fn = reinterpret_cast<EncodeTiled>(p);
+        else
+            cudaGetLastError();
+    });
+    return fn;
+}
 
 int stencil_variant_count(int ndim) { return ndim == 1 ? 3 : 4; }
 const char *stencil_variant_name(int ndim, int v)

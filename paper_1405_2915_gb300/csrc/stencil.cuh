@@ -5,9 +5,17 @@
 // same operations.
 #pragma once
 
+#include <cuda.h>
+
 #include "common.cuh"
 
 namespace skel {
+
+// cuTensorMapEncodeTiled, or nullptr where the driver has none (k_stencil.cu).
+using EncodeTiled = CUresult (*)(CUtensorMap *, CUtensorMapDataType, cuuint32_t, void *, const cuuint64_t *,
+                                 const cuuint64_t *, const cuuint32_t *, const cuuint32_t *, CUtensorMapInterleave,
+                                 CUtensorMapSwizzle, CUtensorMapL2promotion, CUtensorMapFloatOOBfill);
+EncodeTiled encode_tiled();
 
 struct W9 { float w[9]; };
 struct W33 { float w[33]; };

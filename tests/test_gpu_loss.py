@@ -76,6 +76,28 @@ def test_fused_matches_separate_calls(shape, boundary):
     assert np.all(np.abs(to_np(gx) - gs) <= bound + 4 * SUM_REL * suffix)
 
 
+@pytest.mark.parametrize("shape", [(1, 16), (2, 32), (3, 496), (4, 512), (5, 528), (9, 1040), (300, 1024), (7, 8176),
+                                   (1300, 48), (5, 8192)])
+@pytest.mark.parametrize("boundary", ["clamp", "zero"])
+def test_rows_by_tma_match_rows_by_copies(shape, boundary):
+    """Aligned rows of a multiple of 16 columns travel as TMA boxes; the same
+    grid one element off the alignment as 4-byte copies.  The arithmetic of a
+    column is the same, so t and the gradient agree bit for bit; the loss sums
+    its terms in another grouping (float64 above the threads' sums)."""
+    import torch
+    from paper_1405_2915_gb300.autograd import ComposedLossFn
+    x = syn.uniform_f32(9 + shape[1], shape[0] * shape[1], -2.0, 2.0).reshape(shape)
+    res = []
+    for pad in (0, 1):
+        xt = dev_tensor(x, pad).requires_grad_(True)
+        for k in range(3):                       # ring and barriers start afresh on each call
+            L = ComposedLossFn.apply(xt, W_GENERAL, boundary)
+            (gx,) = torch.autograd.grad(L, xt, torch.full_like(L, 1.75))
+        res.append((float(L.detach()), to_np(gx)))
+    assert np.array_equal(res[0][1], res[1][1])
+    assert abs(res[0][0] - res[1][0]) <= SUM_REL * abs(res[1][0])
+
+
 def test_nan_and_infinite_inputs_stay_where_the_definition_puts_them():
     import torch
     from paper_1405_2915_gb300.autograd import composed_loss
