@@ -165,9 +165,10 @@ size_t round256(size_t b) { return (b + 255) & ~(size_t)255; }
 
 bool is_capturing(cudaStream_t stream)
 {
+    if (!stream || stream == cudaStreamLegacy) return false;   // never captured, and asking costs host time
     cudaStreamCaptureStatus st = cudaStreamCaptureStatusNone;
     if (cudaStreamIsCapturing(stream, &st) != cudaSuccess) {
-        cudaGetLastError();   // the legacy stream while another stream captures
+        cudaGetLastError();
         return false;
     }
     return st == cudaStreamCaptureStatusActive;
