@@ -24,14 +24,16 @@
 // planes (plane p holds the p-th group of four columns of every thread, so
 // 16-byte reads are free of bank conflicts) and out by contiguous stores.
 //
-// What bounds it (8192 x 8192): the forward takes 136 us, the backward 176
+// What bounds it (8192 x 8192): the forward takes 127 us, the backward 176
 // (180 and 235 with cp.async), against 79 us each for their HBM traffic
 // (which ncu shows at 1.0 of the algorithmic bytes): instruction issue, which
 // alone takes 80 and 107 us, with 16 warps per SM whose barriers keep them in
 // the same phase (about 50 and 68 instructions per 32 points: two MUFUs and
 // about 15 others of tanhf, 9 FMAs per stencil, 5 to 6 per scan).  The forward
-// computes the next row's tanh beside this row's sums for that reason.  As
-// fifteen separate calls the loss and its gradient took 927 us, here 315.  512
+// therefore splits its barrier into an arrival and a wait, with the stencil's
+// inner columns and the next row's tanh between them (136 us with one whole
+// barrier; the backward, at 128 registers, spills when split so: 209).  As
+// fifteen separate calls the loss and its gradient took 927 us, here 304.  512
 // threads of 16 columns: with 1024 of 8 the scans' shuffles and the edges
 // weigh twice as much.
 //
@@ -67,12 +69,15 @@ __host__ __device__ constexpr int row_floats(int threads) { return C / 4 * plane
 // it touches: o completes the row above, P2 the row itself so far (taps m),
 // P1 the row below; taps in row-major order.
 struct W3 { float w[3]; };
-template <int C>
+// ROW_INNER: the columns that need no neighbour's value; ROW_EDGES: the others.
+enum { ROW_ALL, ROW_INNER, ROW_EDGES };
+template <int PART, int C>
 __device__ __forceinline__ void add_row(const W9 &w, const W3 &m, const float (&e)[C + 2], float (&P1)[C],
                                         float (&P2)[C], float (&o)[C])
 {
 #pragma unroll
     for (int j = 0; j < C; ++j) {
+        if (PART != ROW_ALL && (j == 0 || j == C - 1) != (PART == ROW_EDGES)) continue;
         o[j] = fmaf(w.w[8], e[j + 2], fmaf(w.w[7], e[j + 1], fmaf(w.w[6], e[j], P2[j])));
         P2[j] = fmaf(m.w[2], e[j + 2], fmaf(m.w[1], e[j + 1], fmaf(m.w[0], e[j], P1[j])));
         P1[j] = fmaf(w.w[2], e[j + 2], fmaf(w.w[1], e[j + 1], fmaf(w.w[0], e[j], 0.f)));
@@ -80,11 +85,14 @@ __device__ __forceinline__ void add_row(const W9 &w, const W3 &m, const float (&
 }
 
 // A CLAMP grid's row above row 0 (e: row 0): the sums of row 0 start from it.
-template <int C>
+template <int PART, int C>
 __device__ __forceinline__ void add_row_above(const W9 &w, const float (&e)[C + 2], float (&P1)[C])
 {
 #pragma unroll
-    for (int j = 0; j < C; ++j) P1[j] = fmaf(w.w[2], e[j + 2], fmaf(w.w[1], e[j + 1], fmaf(w.w[0], e[j], 0.f)));
+    for (int j = 0; j < C; ++j) {
+        if (PART != ROW_ALL && (j == 0 || j == C - 1) != (PART == ROW_EDGES)) continue;
+        P1[j] = fmaf(w.w[2], e[j + 2], fmaf(w.w[1], e[j + 1], fmaf(w.w[0], e[j], 0.f)));
+    }
 }
 
 // Inclusive scan of a thread's values in place (groups of four, then the
@@ -346,19 +354,61 @@ struct Exchange {
     float total[kLWarps];                  // scan: the warps' sums
 };
 
-// The columns c-1 and c+C of the row v, from the neighbouring lanes and (ex
-// complete) warps; 0 outside the row.
+// The forward's barrier, in two halves so that work which needs nothing of the
+// other warps stands between them: every warp arrives, later waits until all
+// have.  One mbarrier, one phase per row; the wait is bounded as the copies' is.
+struct BlockSync {
+    uint32_t bar;
+    uint32_t phase;
+    bool ok;
+
+    __device__ __forceinline__ BlockSync(uint64_t *b, int nwarps)   // a __syncthreads follows
+    {
+        bar = (uint32_t)__cvta_generic_to_shared(b);
+        phase = 0;
+        ok = true;
+        if (threadIdx.x == 0) {
+            asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" :: "r"(bar), "r"(nwarps) : "memory");
+            asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+        }
+    }
+    __device__ __forceinline__ void arrive(int lane) const
+    {
+        __syncwarp();
+        if (lane == 0) asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" :: "r"(bar) : "memory");
+    }
+    __device__ __forceinline__ void wait(Control *ctl)
+    {
+        uint32_t done = ok ? 0u : 1u;
+        for (uint32_t it = 0; it < (1u << 22) && !done; ++it)
+            asm volatile("{ .reg .pred p; mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2; selp.u32 %0, 1, 0, p; }"
+                         : "=r"(done) : "r"(bar), "r"(phase) : "memory");
+        phase ^= 1u;
+        if (!done) {
+            ok = false;
+            atomicOr(&ctl->error, kErrTimeout);
+        }
+        __syncwarp();
+    }
+};
+
+// The columns c-1 and c+C of the row v, from the neighbouring lanes; 0 where
+// they are another warp's or outside the row.
 template <int C>
-__device__ __forceinline__ void neighbours(const float (&v)[C], const Exchange &ex, int lane, int warp, int nwarps,
-                                           float (&e)[C + 2])
+__device__ __forceinline__ void neighbours(const float (&v)[C], int lane, float (&e)[C + 2])
 {
-    float l = __shfl_up_sync(0xffffffffu, v[C - 1], 1), r = __shfl_down_sync(0xffffffffu, v[0], 1);
-    if (lane == 0) l = warp > 0 ? ex.last[warp - 1] : 0.f;
-    if (lane == 31) r = warp + 1 < nwarps ? ex.first[warp + 1] : 0.f;
-    e[0] = l;
-    e[C + 1] = r;
+    const float l = __shfl_up_sync(0xffffffffu, v[C - 1], 1), r = __shfl_down_sync(0xffffffffu, v[0], 1);
+    e[0] = lane == 0 ? 0.f : l;
+    e[C + 1] = lane == 31 ? 0.f : r;
 #pragma unroll
     for (int j = 0; j < C; ++j) e[j + 1] = v[j];
+}
+// The same from the neighbouring warps, whose part of ex is complete.
+template <int C>
+__device__ __forceinline__ void warp_neighbours(const Exchange &ex, int lane, int warp, int nwarps, float (&e)[C + 2])
+{
+    if (lane == 0 && warp > 0) e[0] = ex.last[warp - 1];
+    if (lane == 31 && warp + 1 < nwarps) e[C + 1] = ex.first[warp + 1];
 }
 
 // The exclusive form of a warp scan's inclusive value (not wi minus the
@@ -388,6 +438,7 @@ loss_fwd(const __grid_constant__ CUtensorMap tin, const __grid_constant__ CUtens
     constexpr int C = kFwdC;
     extern __shared__ __align__(16) float dyn[];
     __shared__ Exchange ex[2];                // by the row's parity
+    __shared__ uint64_t sync_bar;
     __shared__ double2 red[kLWarps];
     __shared__ int am_last;
     const int64_t r0 = (int64_t)blockIdx.x * H, r1 = r0 + H < rows ? r0 + H : rows;
@@ -396,6 +447,7 @@ loss_fwd(const __grid_constant__ CUtensorMap tin, const __grid_constant__ CUtens
     const int nin = (int)((bottom ? rows : r1 + 1) - q0);
     RowStream<MODE, C, kFwdRing> rs(x, rows, cols, q0, nin, dyn, &tin, &tout, ctl);
     const int lane = rs.lane, warp = rs.warp;
+    BlockSync sync(&sync_bar, rs.nwarps);
     dev::Sum2 su, ss;
     float P1[C], P2[C];
 #pragma unroll
@@ -439,19 +491,25 @@ loss_fwd(const __grid_constant__ CUtensorMap tin, const __grid_constant__ CUtens
             exi.total[warp] = wi;
         }
         rs.template landed<kFwdRing - 3>();   // row i + 1 has landed (its copies by every thread, after the barrier)
-        __syncthreads();
-        neighbours(v, exi, lane, warp, rs.nwarps, e);
+        sync.arrive(lane);
+        neighbours(v, lane, e);
         if (rs.cedge) {
             if (rs.lead) e[0] = clamp ? v[0] : 0.f;
 #pragma unroll
             for (int j = 1; j <= C; ++j)   // the column after the grid's last one
                 if (rs.trail && j == rs.nv) e[j + 1] = clamp ? v[j - 1] : 0.f;
         }
-        // the next row's tanh, independent of this row's sums: the two overlap
-        if (i + 1 < nin) load_t(i + 1, v);
-        if (top && i == 0 && clamp) add_row_above(w, e, P1);   // ZERO: the sums start from 0
+        const bool above = top && i == 0 && clamp;   // ZERO: the sums start from 0
         float o[C];
-        add_row(w, mid, e, P1, P2, o);
+        if (above) add_row_above<ROW_INNER>(w, e, P1);
+        add_row<ROW_INNER>(w, mid, e, P1, P2, o);
+        // the next row's tanh, independent of this row's sums: the two overlap
+        if (MODE == kTma && i + 1 < nin) load_t(i + 1, v);
+        sync.wait(ctl);
+        if (MODE != kTma && i + 1 < nin) load_t(i + 1, v);
+        warp_neighbours<C>(exi, lane, warp, rs.nwarps, e);
+        if (above) add_row_above<ROW_EDGES>(w, e, P1);
+        add_row<ROW_EDGES>(w, mid, e, P1, P2, o);
         if (row > r0) sum_sq(o, su);         // u of row - 1
         if (own) {
             const float base = warp_offset<false>(exi, lane, warp, rs.nwarps) + warp_exclusive<false>(wi, lane);
@@ -467,7 +525,7 @@ loss_fwd(const __grid_constant__ CUtensorMap tin, const __grid_constant__ CUtens
 #pragma unroll
             for (int j = 0; j < C + 2; ++j) e[j] = 0.f;
         }
-        add_row(w, mid, e, P1, P2, o);
+        add_row<ROW_ALL>(w, mid, e, P1, P2, o);
         sum_sq(o, su);
     }
     rs.drain();
@@ -559,7 +617,8 @@ loss_bwd(const __grid_constant__ CUtensorMap tin, const __grid_constant__ CUtens
         if (MODE != kTma) rs.template copy_next<0>();   // into the slot of row i - 3
         // ---- phase 2: u of row - 1, the reverse scan of row - 2 ----
         float e[C + 2];
-        neighbours(v, ex[0], lane, warp, rs.nwarps, e);
+        neighbours(v, lane, e);
+        warp_neighbours<C>(ex[0], lane, warp, rs.nwarps, e);
         if (rs.cedge) {
             if (rs.lead) e[0] = clamp ? v[0] : 0.f;
 #pragma unroll
@@ -567,8 +626,8 @@ loss_bwd(const __grid_constant__ CUtensorMap tin, const __grid_constant__ CUtens
                 if (rs.trail && j == rs.nv) e[j + 1] = clamp ? v[j - 1] : 0.f;
         }
         float u[C];
-        if (row == 0 && clamp) add_row_above(w, e, P1);
-        add_row(w, W3{{w.w[3], w.w[4], w.w[5]}}, e, P1, P2, u);
+        if (row == 0 && clamp) add_row_above<ROW_ALL>(w, e, P1);
+        add_row<ROW_ALL>(w, W3{{w.w[3], w.w[4], w.w[5]}}, e, P1, P2, u);
         if (row >= 1 && row <= rows) {                     // row - 1 is a row of the grid
 #pragma unroll
             for (int j = 0; j < C; ++j) u[j] *= g2;
@@ -599,7 +658,8 @@ loss_bwd(const __grid_constant__ CUtensorMap tin, const __grid_constant__ CUtens
         __syncthreads();
         if (MODE == kTma) rs.template copy_next<0>();   // here: the slot's store has had this row's two phases to end
         // ---- phase 3: the adjoint stencil of row - 2, gx of row - 2 ----
-        neighbours(u, ex[1], lane, warp, rs.nwarps, e);    // 0 outside the grid
+        neighbours(u, lane, e);               // 0 outside the grid
+        warp_neighbours<C>(ex[1], lane, warp, rs.nwarps, e);
         // CLAMP: taps that the forward clamped onto the grid's edge.  The
         // first row also receives what the row above it would, the last row
         // what the row below would: those taps join the middle row's when
@@ -616,7 +676,7 @@ loss_bwd(const __grid_constant__ CUtensorMap tin, const __grid_constant__ CUtens
             for (int k = 0; k < 3; ++k) m.w[k] += wt.w[k];
         }
         float gt[C];
-        add_row(wt, m, e, Q1, Q2, gt);
+        add_row<ROW_ALL>(wt, m, e, Q1, Q2, gt);
         if (clamp && rs.cedge) {
             float ul = 0.f;                   // the thread's last column of the grid
 #pragma unroll
