@@ -308,9 +308,9 @@ int skel_mapoverlap(skel_fn fn, int radius, const float *weights, int nweights,
  * global composition problem; Sec. IV: intermediate results stay on the
  * device).  Variants: per_call (steps single MapOverlap calls, each
  * dispatched as skel_mapoverlap would be) and time_blocked (tile = steps per
- * pass, 1..8: a block stages its tile with that many halo cells and applies
- * the passes' steps in shared memory; CLAMP and ZERO only), which gives the
- * per-call result bit for bit.  in, tmp and out are 2D F32 of one shape and
+ * pass, 1..8: warps stream rows once and keep each step's partial tap sums in
+ * registers; CLAMP and ZERO only), which gives the per-call result bit for
+ * bit.  in, tmp and out are 2D F32 of one shape and
  * pairwise distinct; tmp holds intermediate steps (NULL allowed when steps
  * == 1 or when a single time-blocked pass covers all steps; a variant that
  * needs it then refuses and the call falls back).  in is not modified.
