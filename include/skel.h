@@ -137,14 +137,17 @@ const char *skel_last_error(void);
  * free(ptr, stream, ctx) releases it (stream-ordered).  Passing NULL for
  * alloc restores the built-in allocator (cudaMallocFromPoolAsync on the library's own pool / cudaFreeAsync).
  * Containers and scratch already allocated keep the allocator they were
- * allocated with.  Not thread-safe against concurrent skeleton calls. */
+ * allocated with; the scratch of calls captured into a CUDA graph always
+ * comes from the built-in one.  Not thread-safe against concurrent skeleton calls. */
 int skel_set_allocator(void *(*alloc)(size_t bytes, void *stream, void *ctx),
                        void (*free_fn)(void *ptr, void *stream, void *ctx), void *ctx);
 
 /* Releases the cached scratch memory and result slots of every stream, and
  * returns the unused memory of the built-in allocator's pools (the library
  * keeps its own pool per device, which holds freed memory for later calls).
- * Containers are not touched.  Waits for the streams that used them. */
+ * Containers are not touched, nor is the scratch of calls captured into a
+ * CUDA graph that still exists (it goes with the last graph that holds it).
+ * Waits for the streams that used them. */
 int skel_release_cached(void);
 
 /* Number of CUDA kernels the library has launched in this process (all
@@ -510,7 +513,7 @@ const char *skel_variant_name(int skeleton, int variant);
 /* ---------------------------------------------------- device status ---- */
 
 /* Waits for `stream` and reports device-side failures of the calls made on
- * it since the last check (and of skel_scan_noalloc calls on the current
+ * it, and in replays of the graphs captured on it, since the last check (and of skel_scan_noalloc calls on the current
  * device, whose status sits in its static array): SKEL_ERR_TIMEOUT if a
  * bounded wait (the scan's look-back over predecessor tiles, a TMA copy)
  * gave up, SKEL_ERR_INVALID_ARG

@@ -1690,13 +1690,11 @@ int skel_check_device(void *stream)
         cudaStream_t s = (cudaStream_t)stream;
         SKEL_CUDA_TRY(cudaStreamSynchronize(s));
         uint32_t err = 0;
-        if (Control *ctl = scratch_control(s)) {
-            SKEL_CUDA_TRY(cudaMemcpy(&err, &ctl->error, sizeof(err), cudaMemcpyDeviceToHost));
-            if (err) SKEL_CUDA_TRY(cudaMemset(&ctl->error, 0, sizeof(uint32_t)));
-        }
+        int rc = scratch_take_status(s, &err);
+        if (rc) return rc;
         // the allocation-free scan records into its own static control block
         uint32_t err_static = 0;
-        int rc = noalloc_take_status(&err_static);
+        rc = noalloc_take_status(&err_static);
         if (rc) return rc;
         err |= err_static;
         if (err) {

@@ -103,11 +103,15 @@ constexpr uint32_t kMaxEpoch = 255;
 // `word_count` descriptor words.  Scratch is cached per (device, stream) and
 // reused by later calls on the same stream (stream order serialises them).
 // A call asking for words gets a fresh epoch (the words are cleared when the
-// epoch counter wraps or the region grows).
+// epoch counter wraps or the region grows).  On a stream that is being
+// captured the scratch belongs to the capture's graph: a replay shares none of
+// it with other calls, and a node before each call that asks for words clears
+// them (the epoch is 1).
 int get_scratch(cudaStream_t stream, size_t data_bytes, size_t word_count, Scratch *out);
 
-// Control block of the scratch of `stream`, or nullptr if none was made.
-Control *scratch_control(cudaStream_t stream);
+// Device status bits recorded in the scratch of `stream` and of the graphs
+// captured on it (current device).  Clears them.  Synchronous.
+int scratch_take_status(cudaStream_t stream, uint32_t *err);
 int release_scratch();
 // Device status bits recorded by the allocation-free scan on the current
 // device (its control block lives in a static array, not in a stream's

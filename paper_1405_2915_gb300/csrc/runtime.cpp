@@ -7,11 +7,13 @@
 #include <array>
 #include <atomic>
 #include <cmath>
+#include <cstddef>
 #include <cstdio>
 #include <cstring>
 #include <fstream>
 #include <map>
 #include <mutex>
+#include <set>
 #include <sstream>
 #include <string>
 #include <tuple>
@@ -149,49 +151,136 @@ struct ScratchBlock {
     size_t data_cap = 0;    // bytes
     uint32_t epoch = 0;
     Allocator alloc{};
-    bool captured = false;  // a graph captured on the stream may hold its address
 };
-struct RetiredBlock {
-    int dev;
-    cudaStream_t stream;
-    void *base;
-    Allocator alloc;
-};
-std::vector<RetiredBlock> g_retired;   // replaced blocks that a graph may hold; freed by skel_release_cached
 std::mutex g_scr_mu;
 std::map<std::pair<int, cudaStream_t>, ScratchBlock> g_scratch;
 
+// Scratch of the calls that one stream capture records on one stream.  A
+// graph is replayed at any time and on any stream, so its calls share no
+// memory with the stream's later calls or with another graph: a counter or a
+// partial result of one would be the other's.  The graph, and what is
+// instantiated from it, owns a reference to the block; once the last one is
+// gone the next capture or skel_release_cached frees the memory.
+struct GraphBlock {
+    int dev;
+    cudaStream_t stream;
+    unsigned long long capture;         // the capture's id
+    void *base;
+    size_t word_cap, data_cap;
+    std::atomic<bool> unused{false};    // no graph holds it any more
+};
+
+// Never destroyed: a graph may be destroyed after the library's static data.
+std::vector<GraphBlock *> &graph_blocks()
+{
+    static auto *blocks = new std::vector<GraphBlock *>();
+    return *blocks;
+}
+
 size_t round256(size_t b) { return (b + 255) & ~(size_t)255; }
 
-bool is_capturing(cudaStream_t stream)
+// Whether `stream` is being captured, and into which graph.
+bool capture_of(cudaStream_t stream, unsigned long long *id, cudaGraph_t *graph)
 {
     if (!stream || stream == cudaStreamLegacy) return false;   // never captured, and asking costs host time
     cudaStreamCaptureStatus st = cudaStreamCaptureStatusNone;
-    if (cudaStreamIsCapturing(stream, &st) != cudaSuccess) {
+    cudaError_t e = cudaStreamIsCapturing(stream, &st);
+    if (e == cudaSuccess && st == cudaStreamCaptureStatusActive)
+        e = cudaStreamGetCaptureInfo(stream, &st, id, graph, nullptr, nullptr, nullptr);
+    if (e != cudaSuccess) {
         cudaGetLastError();
         return false;
     }
     return st == cudaStreamCaptureStatusActive;
 }
 
-// Zeroed memory for a block that `stream` needs while it is being captured:
-// made on a stream of its own, so that it is neither a node of the graph nor
-// bound to its lifetime.
-void *alloc_beside_capture(size_t bytes)
+// Frees the blocks of device dev that no graph holds, on `stream`.
+void free_unused_blocks(int dev, cudaStream_t stream)
 {
+    auto &v = graph_blocks();
+    for (size_t k = 0; k < v.size();) {
+        if (v[k]->dev != dev || !v[k]->unused.load(std::memory_order_acquire)) {
+            ++k;
+            continue;
+        }
+        dev_free(Allocator{nullptr, nullptr, nullptr}, v[k]->base, stream);
+        delete v[k];
+        v[k] = v.back();
+        v.pop_back();
+    }
+}
+
+// Zeroed memory for a stream that is being captured: made on a stream of its
+// own, so that the allocation is not a node of the graph.
+void *alloc_beside_capture(int dev, size_t bytes)
+{
+    const Allocator own{nullptr, nullptr, nullptr};
     cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;
     if (cudaThreadExchangeStreamCaptureMode(&mode) != cudaSuccess) return nullptr;
     void *p = nullptr;
     cudaStream_t side;
     if (cudaStreamCreateWithFlags(&side, cudaStreamNonBlocking) == cudaSuccess) {
-        p = dev_alloc(Allocator{nullptr, nullptr, nullptr}, bytes, side);
-        if (p && cudaMemsetAsync(p, 0, bytes, side) != cudaSuccess) p = nullptr;
+        free_unused_blocks(dev, side);
+        p = dev_alloc(own, bytes, side);
+        const bool ok = p && cudaMemsetAsync(p, 0, bytes, side) == cudaSuccess;
+        if (p && !ok) {
+            dev_free(own, p, side);
+            p = nullptr;
+        }
         if (cudaStreamSynchronize(side) != cudaSuccess) p = nullptr;
         cudaStreamDestroy(side);
     }
     cudaGetLastError();
     cudaThreadExchangeStreamCaptureMode(&mode);
     return p;
+}
+
+void CUDART_CB graph_gone(void *block)   // no CUDA calls and no locks in here
+{
+    static_cast<GraphBlock *>(block)->unused.store(true, std::memory_order_release);
+}
+
+// get_scratch for a stream that is being captured.  A replay's look-back
+// words must start cleared: the tag is a launch parameter, the same in every
+// replay, and would mark the last replay's words as this one's.
+int capture_scratch(int dev, cudaStream_t stream, unsigned long long id, cudaGraph_t graph, size_t data_bytes,
+                    size_t word_count, Scratch *out)
+{
+    GraphBlock *b = nullptr;
+    for (GraphBlock *k : graph_blocks())
+        if (k->dev == dev && k->stream == stream && k->capture == id && !k->unused.load(std::memory_order_acquire) &&
+            data_bytes <= k->data_cap && word_count <= k->word_cap)
+            b = k;
+    if (!b) {
+        const size_t wc = std::max<size_t>(round256(word_count * 8) / 8, 32), dc = std::max<size_t>(round256(data_bytes), 256);
+        void *base = alloc_beside_capture(dev, sizeof(Control) + wc * 8 + dc);
+        if (!base) return fail(SKEL_ERR_OOM, "scratch allocation failed");
+        b = new GraphBlock{dev, stream, id, base, wc, dc};
+        graph_blocks().push_back(b);
+        cudaUserObject_t owner;
+        cudaError_t e = cudaUserObjectCreate(&owner, b, graph_gone, 1, cudaUserObjectNoDestructorSync);
+        if (e != cudaSuccess) {
+            b->unused = true;
+            return fail_cuda(e, "scratch of a captured call");
+        }
+        e = cudaGraphRetainUserObject(graph, owner, 1, cudaGraphUserObjectMove);
+        if (e != cudaSuccess) {
+            cudaUserObjectRelease(owner, 1);   // runs graph_gone
+            return fail_cuda(e, "scratch of a captured call");
+        }
+    }
+    unsigned char *base = static_cast<unsigned char *>(b->base);
+    out->ctl = reinterpret_cast<Control *>(base);
+    out->words = reinterpret_cast<uint64_t *>(base + sizeof(Control));
+    out->data = base + sizeof(Control) + b->word_cap * 8;
+    out->data_bytes = b->data_cap;
+    out->epoch = 1;
+    if (word_count > 0) {   // one node: the control words from `abort` on, and the look-back words behind them
+        const size_t skip = offsetof(Control, abort);
+        cudaError_t e = cudaMemsetAsync(base + skip, 0, sizeof(Control) - skip + word_count * 8, stream);
+        if (e != cudaSuccess) return fail_cuda(e, "look-back word clear");
+    }
+    return SKEL_OK;
 }
 }  // namespace
 
@@ -200,11 +289,11 @@ int get_scratch(cudaStream_t stream, size_t data_bytes, size_t word_count, Scrat
     int dev = 0;
     cudaGetDevice(&dev);
     std::lock_guard<std::mutex> lk(g_scr_mu);
+    unsigned long long id = 0;
+    cudaGraph_t graph = nullptr;
+    if (capture_of(stream, &id, &graph)) return capture_scratch(dev, stream, id, graph, data_bytes, word_count, out);
     ScratchBlock &b = g_scratch[{dev, stream}];
     const bool grow = !b.base || data_bytes > b.data_cap || word_count > b.word_cap;
-    // a block whose address a captured graph holds is kept when a larger one
-    // replaces it: a replay still uses it
-    const bool capturing = is_capturing(stream);
     if (grow) {
         size_t wc = std::max(word_count, b.word_cap);
         size_t dc = std::max(data_bytes, b.data_cap);
@@ -215,12 +304,10 @@ int get_scratch(cudaStream_t stream, size_t data_bytes, size_t word_count, Scrat
         }
         wc = std::max<size_t>(round256(wc * 8) / 8, 32);
         dc = std::max<size_t>(round256(dc), 256);
-        if (b.base && (b.captured || capturing)) g_retired.push_back(RetiredBlock{dev, stream, b.base, b.alloc});
-        else if (b.base) dev_free(b.alloc, b.base, stream);
-        b.captured = false;
-        b.alloc = capturing ? Allocator{nullptr, nullptr, nullptr} : current_allocator();
+        if (b.base) dev_free(b.alloc, b.base, stream);
+        b.alloc = current_allocator();
         const size_t total = sizeof(Control) + wc * 8 + dc;
-        b.base = capturing ? alloc_beside_capture(total) : dev_alloc(b.alloc, total, stream);
+        b.base = dev_alloc(b.alloc, total, stream);
         if (!b.base) {
             b = ScratchBlock{};
             return fail(SKEL_ERR_OOM, "scratch allocation failed");
@@ -228,12 +315,9 @@ int get_scratch(cudaStream_t stream, size_t data_bytes, size_t word_count, Scrat
         b.word_cap = wc;
         b.data_cap = dc;
         b.epoch = 0;
-        if (!capturing) {
-            cudaError_t e = cudaMemsetAsync(b.base, 0, total, stream);
-            if (e != cudaSuccess) return fail_cuda(e, "scratch clear");
-        }
+        cudaError_t e = cudaMemsetAsync(b.base, 0, total, stream);
+        if (e != cudaSuccess) return fail_cuda(e, "scratch clear");
     }
-    b.captured |= capturing;
     unsigned char *base = static_cast<unsigned char *>(b.base);
     out->ctl = reinterpret_cast<Control *>(base);
     out->words = reinterpret_cast<uint64_t *>(base + sizeof(Control));
@@ -317,16 +401,26 @@ HostSlot::~HostSlot()
     g_hslot_used &= ~(uint64_t(1) << index);
 }
 
-// Device-side status words of the scratch of `stream` (current device), or
-// nullptr if the stream never used scratch.
-Control *scratch_control(cudaStream_t stream)
+// Device status bits of the scratch of `stream` and of the graphs captured on
+// it (current device); clears them.  Synchronous.
+int scratch_take_status(cudaStream_t stream, uint32_t *err)
 {
     int dev = 0;
     cudaGetDevice(&dev);
+    *err = 0;
     std::lock_guard<std::mutex> lk(g_scr_mu);
-    auto it = g_scratch.find({dev, stream});
-    if (it == g_scratch.end() || !it->second.base) return nullptr;
-    return reinterpret_cast<Control *>(it->second.base);
+    std::vector<void *> bases;
+    const auto it = g_scratch.find({dev, stream});
+    if (it != g_scratch.end() && it->second.base) bases.push_back(it->second.base);
+    for (const GraphBlock *b : graph_blocks())
+        if (b->dev == dev && b->stream == stream) bases.push_back(b->base);
+    for (void *base : bases) {
+        uint32_t *word = &static_cast<Control *>(base)->error, bits = 0;
+        SKEL_CUDA_TRY(cudaMemcpy(&bits, word, sizeof(bits), cudaMemcpyDeviceToHost));
+        if (bits) SKEL_CUDA_TRY(cudaMemset(word, 0, sizeof(bits)));
+        *err |= bits;
+    }
+    return SKEL_OK;
 }
 
 int release_scratch()
@@ -346,14 +440,13 @@ int release_scratch()
         cudaStreamSynchronize(kv.first.second);
         dev_free(kv.second.second, kv.second.first, kv.first.second);
     }
-    cudaSetDevice(cur);
-    for (const RetiredBlock &r : g_retired) {
-        cudaSetDevice(r.dev);
-        cudaStreamSynchronize(r.stream);
-        dev_free(r.alloc, r.base, r.stream);
+    std::set<int> devs;
+    for (const GraphBlock *b : graph_blocks()) devs.insert(b->dev);
+    for (int d : devs) {
+        cudaSetDevice(d);
+        free_unused_blocks(d, nullptr);
     }
     cudaSetDevice(cur);
-    g_retired.clear();
     g_scratch.clear();
     g_slots.clear();
     {
