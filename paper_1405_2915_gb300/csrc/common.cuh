@@ -81,17 +81,22 @@ __device__ __forceinline__ void cp_commit() { asm volatile("cp.async.commit_grou
 template <int N>
 __device__ __forceinline__ void cp_wait() { asm volatile("cp.async.wait_group %0;" :: "n"(N) : "memory"); }
 
-// A float32 sum and the rounding errors it made, each exact (Knuth's TwoSum).
+// A running float32 sum hi + lo: lo holds the rounding errors of hi, each
+// exact (Knuth's TwoSum), about 48 bits together with float32 operations only
+// (float64 units are few on this GPU).  The error term of an infinite sum is
+// inf - inf, so lo is read through low(), which is 0 there.
 struct Sum2 {
     float hi = 0.f, lo = 0.f;
+    Sum2() = default;
+    __device__ __forceinline__ explicit Sum2(double v) : hi((float)v), lo((float)(v - (double)(float)v)) {}
     __device__ __forceinline__ void add(float v)
     {
         const float s = hi + v, bv = s - hi;
         lo += (hi - (s - bv)) + (v - bv);
         hi = s;
     }
-    // an infinite sum has no meaningful error term
-    __device__ __forceinline__ double value() const { return isinf(hi) ? (double)hi : (double)hi + (double)lo; }
+    __device__ __forceinline__ float low() const { return isinf(hi) ? 0.f : lo; }
+    __device__ __forceinline__ double value() const { return (double)hi + (double)low(); }
 };
 
 // The first statement of every kernel.  launch_kernel lets a kernel's blocks

@@ -45,9 +45,7 @@ constexpr int kUnit = 128;                       // elements per warp scan
 constexpr int kWaveMaxWarps = 32;
 constexpr int kWaveMaxUnits = 432;               // 55296 elements, 216 KiB of shared memory per block
 
-// A running sum hi + lo of elements.  float32: lo holds the rounding errors of
-// hi, each exact (Knuth's TwoSum), about 48 bits together with float32
-// operations only (float64 units are few on this GPU).
+// A running sum of elements: float32 as dev::Sum2, integers as they are.
 template <class T> struct Run;
 template <> struct Run<uint32_t> {
     uint32_t hi;
@@ -55,20 +53,12 @@ template <> struct Run<uint32_t> {
     __device__ __forceinline__ Run() : hi(0u) {}
     __device__ __forceinline__ explicit Run(uint32_t v) : hi(v) {}
     __device__ __forceinline__ void add(uint32_t v) { hi += v; }
+    __device__ __forceinline__ uint32_t low() const { return 0u; }
     __device__ __forceinline__ uint32_t value() const { return hi; }
 };
-template <> struct Run<float> {
-    float hi, lo;
-    __device__ __forceinline__ Run() : hi(0.f), lo(0.f) {}
-    __device__ __forceinline__ explicit Run(double v) : hi((float)v), lo((float)(v - (double)(float)v)) {}
-    __device__ __forceinline__ void add(float v)
-    {
-        const float s = hi + v, bv = s - hi;
-        lo += (hi - (s - bv)) + (v - bv);
-        hi = s;
-    }
-    // an infinite sum has no meaningful error term
-    __device__ __forceinline__ double value() const { return isinf(hi) ? (double)hi : (double)hi + (double)lo; }
+template <> struct Run<float> : dev::Sum2 {
+    Run() = default;
+    __device__ __forceinline__ explicit Run(double v) : dev::Sum2(v) {}
 };
 __device__ __forceinline__ void set_lo(Run<uint32_t> &, uint32_t) {}
 __device__ __forceinline__ void set_lo(Run<float> &r, float lo) { r.lo = lo; }
@@ -88,7 +78,7 @@ __device__ __forceinline__ Run<float> warp_total(Run<float> r)
     return r;
 }
 
-// Sum over lanes of the running type, by shuffles.
+// Shuffles of the carry type.
 __device__ __forceinline__ uint32_t shfl_up_ct(uint32_t v, int d) { return __shfl_up_sync(0xffffffffu, v, d); }
 __device__ __forceinline__ double shfl_up_ct(double v, int d) { return __shfl_up_sync(0xffffffffu, v, d); }
 
@@ -240,7 +230,7 @@ scan_wave(const T *__restrict__ in, T *__restrict__ out, WaveGeom g, uint64_t *_
     // N units from number i on: interleaved warp scans, then the stores
     auto scan_units = [&](int i, auto n_t) {
         constexpr int N = decltype(n_t)::value;
-        const T hi = carry.hi, lo = carry.lo;
+        const T hi = carry.hi, lo = carry.low();
         T loc = T(0);
         V4 o[N];
 #pragma unroll
