@@ -159,6 +159,14 @@ __device__ __forceinline__ T warp_incl_scan_add(T v)
     }
     return v;
 }
+// Its exclusive form, from the lane before (the inclusive value minus the
+// lane's own is NaN where that is infinite).
+template <class T>
+__device__ __forceinline__ T warp_exclusive(T incl)
+{
+    const T t = __shfl_up_sync(0xffffffffu, incl, 1);
+    return (threadIdx.x & 31) == 0 ? T(0) : t;
+}
 
 // ----------------------------------------------------------- map functors --
 // out = f(x, y; a), one instantiation per skel_fn (the compiled-in user

@@ -1302,17 +1302,16 @@ scan_tile_prefixes(CT *__restrict__ sums, int64_t tps)
             v[i] = j < tps ? s[j] : CT(0);
             t = t + v[i];
         }
-        CT wi = dev::warp_incl_scan_add(t);
+        const CT wi = dev::warp_incl_scan_add(t), wx = dev::warp_exclusive(wi);
         if (lane == 31) smem[w] = wi;
         __syncthreads();
         if (w == 0) {
-            CT a = smem[lane];
-            CT ai = dev::warp_incl_scan_add(a);
-            smem[lane] = ai - a;   // exact for integers; float64 rounding far below float32 output
+            const CT ai = dev::warp_incl_scan_add(smem[lane]), ax = dev::warp_exclusive(ai);
+            smem[lane] = ax;
             if (lane == 31) smem[32] = ai;
         }
         __syncthreads();
-        CT run = carry + smem[w] + (wi - t);
+        CT run = carry + smem[w] + wx;
 #pragma unroll
         for (int i = 0; i < IPT; ++i) {
             const int64_t j = c0 + (int64_t)threadIdx.x * IPT + i;

@@ -91,16 +91,9 @@ template <> struct RrCarry<uint32_t> {
     __device__ __forceinline__ uint32_t base() const { return c; }
     __device__ __forceinline__ void add(uint32_t v) { c += v; }
 };
-template <> struct RrCarry<float> {
-    float hi, lo;
-    __device__ __forceinline__ explicit RrCarry(double e) : hi((float)e), lo((float)(e - (double)(float)e)) {}
-    __device__ __forceinline__ float base() const { return hi + lo; }
-    __device__ __forceinline__ void add(float v)
-    {
-        const float s = hi + v, bv = s - hi;
-        lo += (hi - (s - bv)) + (v - bv);   // the rounding error of hi + v, exactly
-        hi = s;
-    }
+template <> struct RrCarry<float> : dev::Sum2 {
+    __device__ __forceinline__ explicit RrCarry(double e) : dev::Sum2(e) {}
+    __device__ __forceinline__ float base() const { return hi + low(); }
 };
 
 template <class T, bool INCL, bool REV, bool ROWS, int R, int NC>

@@ -8,7 +8,7 @@ from helpers import SUM_REL, dev_empty, dev_tensor, forced, skel, to_np, wrap
 
 pytestmark = pytest.mark.gpu
 
-VARIANTS = [9]
+VARIANTS = list(range(10))
 SHAPES = [(300_003,), (5_000_012,), (3, 55_296), (7, 8191), (90, 257), (5, 130)]
 INF, NAN = np.float32(np.inf), np.float32(np.nan)
 # values at fractions of the sequence (of every second row)
