@@ -42,7 +42,31 @@ __device__ __forceinline__ Seg warp_seg_scan(Seg v)
     }
     return v;
 }
-
+// N warp scans at once: inc the inclusive sums of the lanes' values v, ex the
+// exclusive ones.  ex is summed on the way: inc minus v loses what v swamps,
+// and is NaN where v is infinite; a shuffle from the lane before takes longer
+// (variant 7, 4096 instances of 64 to 2^20: 708 us, 726 by shuffles, 705 by
+// the difference).
+template <int N>
+__device__ __forceinline__ void warp_scans(const float (&v)[N], float (&inc)[N], float (&ex)[N])
+{
+    const int lane = threadIdx.x & 31;
+#pragma unroll
+    for (int k = 0; k < N; ++k) {
+        inc[k] = v[k];
+        ex[k] = 0.f;
+    }
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1)
+#pragma unroll
+        for (int k = 0; k < N; ++k) {
+            const float u = __shfl_up_sync(0xffffffffu, inc[k], o);
+            if (lane >= o) {
+                ex[k] += u;
+                inc[k] += u;
+            }
+        }
+}
 
 }  // namespace
 }  // namespace skel

@@ -665,8 +665,8 @@ batched_rts_prefix(Layout L, int64_t B, const double *__restrict__ aggS, const d
             const int64_t k = k0 + lane;
             const double a = (scan && k < s1) ? aggS[k] : 0.0;
             if (red && k < s1) q += aggQ[k];
-            const double incl = dev::warp_incl_scan_add(a);
-            if (scan && k < s1) prefS[k] = carry + (incl - a);
+            const double incl = dev::warp_incl_scan_add(a), excl = dev::warp_exclusive(incl);
+            if (scan && k < s1) prefS[k] = carry + excl;
             carry += __shfl_sync(0xffffffffu, incl, 31);
         }
         if (red) {

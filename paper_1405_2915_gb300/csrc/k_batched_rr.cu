@@ -61,19 +61,11 @@ __device__ __forceinline__ void br_expect(uint64_t *bar, uint32_t bytes)
     asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" :: "r"(smem_u32(bar)), "r"(bytes) : "memory");
 }
 
-// A running float32 sum kept as an unevaluated pair hi + lo and advanced by
-// an exact two-sum (Knuth's TwoSum): about 48 bits with float32 operations.
-struct BrFF {
-    float hi, lo;
-    __device__ __forceinline__ float base() const { return hi + lo; }
+// A running float32 sum of a tile (about 48 bits, as dev::Sum2 keeps them).
+struct BrFF : dev::Sum2 {
+    __device__ __forceinline__ float base() const { return hi + low(); }
     __device__ __forceinline__ void set(float v) { hi = v; lo = 0.f; }
-    __device__ __forceinline__ void set(double v) { hi = (float)v; lo = (float)(v - (double)hi); }
-    __device__ __forceinline__ void add(float v)
-    {
-        const float s = hi + v, bv = s - hi;
-        lo += (hi - (s - bv)) + (v - bv);
-        hi = s;
-    }
+    __device__ __forceinline__ void set(double v) { *static_cast<dev::Sum2 *>(this) = dev::Sum2(v); }
 };
 
 // Checks the offsets and writes each tile's placement, one warp per instance:
@@ -437,16 +429,12 @@ batched_br(const float *__restrict__ values, const int64_t *__restrict__ off, in
                 h5 = x & 31u;
             }
             if (!__any_sync(0xffffffffu, h5 != 0u)) {   // no start and no end among these 128: a plain scan
-                const float a = v.x, ab = a + v.y, abc = ab + v.z, mine = abc + v.w;
-                float inc = mine;
-#pragma unroll
-                for (int o = 1; o < 32; o <<= 1) {
-                    const float u = __shfl_up_sync(0xffffffffu, inc, o);
-                    if (lane >= o) inc += u;
-                }
+                const float a = v.x, ab = a + v.y, abc = ab + v.z, mine[1] = {abc + v.w};
+                float inc[1], ex[1];
+                warp_scans(mine, inc, ex);
                 if (SCAN) {
-                    const float run = cs.base() + (inc - mine);
-                    const float4 o4 = INCL ? make_float4(run + a, run + ab, run + abc, run + mine)
+                    const float run = cs.base() + ex[0];
+                    const float4 o4 = INCL ? make_float4(run + a, run + ab, run + abc, run + mine[0])
                                            : make_float4(run, run + a, run + ab, run + abc);
                     if (t < nfull) dev::st_stream(reinterpret_cast<float4 *>(scan_out + t0) + g * 32 + lane, o4);
                     else {
@@ -456,7 +444,7 @@ batched_br(const float *__restrict__ values, const int64_t *__restrict__ off, in
                             if (e + i < len) scan_out[t0 + e + i] = o[i];
                     }
                 }
-                cs.add(__shfl_sync(0xffffffffu, inc, 31));
+                cs.add(__shfl_sync(0xffffffffu, inc[0], 31));
                 if (ends) {   // the squares run on to an instance end later in the tile
                     float q = fmaf(v.x, v.x, v.y * v.y) + fmaf(v.z, v.z, v.w * v.w);
 #pragma unroll
@@ -522,7 +510,7 @@ batched_br(const float *__restrict__ values, const int64_t *__restrict__ off, in
                 continue;
             }
             float4 v[4];
-            float a[4], ab[4], abc[4], mine[4], inc[4];
+            float a[4], ab[4], abc[4], mine[4], inc[4], ex[4];
 #pragma unroll
             for (int k = 0; k < 4; ++k) {
                 v[k] = src[(4 * g4 + k) * 32 + lane];
@@ -530,21 +518,14 @@ batched_br(const float *__restrict__ values, const int64_t *__restrict__ off, in
                 ab[k] = a[k] + v[k].y;
                 abc[k] = ab[k] + v[k].z;
                 mine[k] = abc[k] + v[k].w;
-                inc[k] = mine[k];
             }
-#pragma unroll
-            for (int o = 1; o < 32; o <<= 1)
-#pragma unroll
-                for (int k = 0; k < 4; ++k) {
-                    const float u = __shfl_up_sync(0xffffffffu, inc[k], o);
-                    if (lane >= o) inc[k] += u;
-                }
+            warp_scans(mine, inc, ex);
             const float base = cs.base();
             float loc = 0.f;
 #pragma unroll
             for (int k = 0; k < 4; ++k) {
                 if (SCAN) {
-                    const float run = base + (loc + (inc[k] - mine[k]));
+                    const float run = base + (loc + ex[k]);
                     const float4 o4 = INCL ? make_float4(run + a[k], run + ab[k], run + abc[k], run + mine[k])
                                            : make_float4(run, run + a[k], run + ab[k], run + abc[k]);
                     dev::st_stream(reinterpret_cast<float4 *>(scan_out + t0) + (4 * g4 + k) * 32 + lane, o4);

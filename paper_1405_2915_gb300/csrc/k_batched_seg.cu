@@ -317,23 +317,15 @@ batched_seg(const float *__restrict__ values, const int64_t *__restrict__ off, i
         if (!SCAN && head_free(j)) return;   // nothing to store and no instance ends here
         if (SCAN && head_free(j)) {   // a plain scan of the sums; no instance ends here, so no squares are needed
             // the four 128-element blocks' warp scans interleaved, then their carries chained
-            float a[4], ab[4], abc[4], mine[4], inc[4];
+            float a[4], ab[4], abc[4], mine[4], inc[4], ex[4];
 #pragma unroll
             for (int k = 0; k < 4; ++k) {
                 a[k] = v[k].x;
                 ab[k] = a[k] + v[k].y;
                 abc[k] = ab[k] + v[k].z;
                 mine[k] = abc[k] + v[k].w;
-                inc[k] = mine[k];
             }
-#pragma unroll
-            for (int o = 1; o < 32; o <<= 1) {
-#pragma unroll
-                for (int k = 0; k < 4; ++k) {
-                    const float u = __shfl_up_sync(0xffffffffu, inc[k], o);
-                    if (lane >= o) inc[k] += u;
-                }
-            }
+            warp_scans(mine, inc, ex);
             float base[4];
             base[0] = c.s;
 #pragma unroll
@@ -341,7 +333,7 @@ batched_seg(const float *__restrict__ values, const int64_t *__restrict__ off, i
 #pragma unroll
             for (int k = 0; k < 4; ++k) {
                 const int e = j * kSubTile + w * 512 + k * 128 + lane * 4;
-                const float run = base[k] + (inc[k] - mine[k]);
+                const float run = base[k] + ex[k];
                 const float4 o4 = INCL ? make_float4(run + a[k], run + ab[k], run + abc[k], run + mine[k])
                                        : make_float4(run, run + a[k], run + ab[k], run + abc[k]);
                 if (!PART || e + 3 < len) {
@@ -361,15 +353,11 @@ batched_seg(const float *__restrict__ values, const int64_t *__restrict__ off, i
             const uint32_t hb = head4(e);
             if (!__any_sync(0xffffffffu, hb)) {   // no head and no instance end among these 128: a plain scan
                 if (SCAN) {
-                    const float a = v[k].x, ab = a + v[k].y, abc = ab + v[k].z, mine = abc + v[k].w;
-                    float inc = mine;
-#pragma unroll
-                    for (int o = 1; o < 32; o <<= 1) {
-                        const float u = __shfl_up_sync(0xffffffffu, inc, o);
-                        if (lane >= o) inc += u;
-                    }
-                    const float run = c.s + (inc - mine);
-                    const float4 o4 = INCL ? make_float4(run + a, run + ab, run + abc, run + mine)
+                    const float a = v[k].x, ab = a + v[k].y, abc = ab + v[k].z, mine[1] = {abc + v[k].w};
+                    float inc[1], ex[1];
+                    warp_scans(mine, inc, ex);
+                    const float run = c.s + ex[0];
+                    const float4 o4 = INCL ? make_float4(run + a, run + ab, run + abc, run + mine[0])
                                            : make_float4(run, run + a, run + ab, run + abc);
                     if (!PART || e + 3 < len) {
                         dev::st_stream(reinterpret_cast<float4 *>(scan_out + t0 + e), o4);
@@ -379,7 +367,7 @@ batched_seg(const float *__restrict__ values, const int64_t *__restrict__ off, i
                         for (int i = 0; i < 4; ++i)
                             if (e + i < len) scan_out[t0 + e + i] = o[i];
                     }
-                    c.s += __shfl_sync(0xffffffffu, inc, 31);
+                    c.s += __shfl_sync(0xffffffffu, inc[0], 31);
                 }
                 if (RED) {   // the squares run on to an instance end later in the range
                     float q = fmaf(v[k].x, v[k].x, fmaf(v[k].y, v[k].y, fmaf(v[k].z, v[k].z, v[k].w * v[k].w)));

@@ -1,4 +1,4 @@
-"""Scans over infinities, infinities of both signs, NaN and sums that leave
+"""Scans (also of batched instances) over infinities, infinities of both signs, NaN and sums that leave
 float32's range: the outputs are infinite and NaN exactly where the prefix sums
 in 64 bits, rounded to float32, are."""
 import numpy as np
@@ -67,3 +67,49 @@ def test_scan(variant, shape, pattern):
                 special = ~np.isfinite(rounded)
                 assert np.array_equal(got[special], rounded[special], equal_nan=True)
                 assert np.all(np.abs(got[~special] - want[~special]) <= SUM_REL * mag[~special])
+
+
+LENS = [5, 300_003, 0, 4096, 130, 8191, 1, 70_000]
+
+
+@pytest.mark.parametrize("variant,tile", [(0, 0), (1, 0), (2, 0), (3, 0), (4, 0), (5, 0), (6, 0), (6, 1), (7, 0), (7, 1)])
+@pytest.mark.parametrize("pattern", PATTERNS)
+def test_batched(variant, tile, pattern):
+    """The pattern in every second instance; the others stay finite."""
+    import torch
+    sk = skel()
+    parts = [sequence((n,), pattern) if k % 2 and n else np.ones(n, np.float32) for k, n in enumerate(LENS)]
+    off = np.concatenate([[0], np.cumsum(LENS)]).astype(np.int64)
+    cv, co = wrap(dev_tensor(np.concatenate(parts))), wrap(dev_tensor(off))
+    res, out = dev_empty((len(LENS),), torch.float32), dev_empty((int(off[-1]),), torch.float32)
+    for inclusive in (True, False):
+        with forced("batched", variant, 0, 4, tile):
+            sk.skel_batched(cv, co, wrap(res), wrap(out), inclusive)
+        sums, got = to_np(res).copy(), to_np(out).copy()
+        for k, x in enumerate(parts):
+            want, mag = prefixes(x, inclusive, False)
+            g = got[off[k]:off[k + 1]]
+            with np.errstate(all="ignore"):
+                rounded = want.astype(np.float32)
+                special = ~np.isfinite(rounded)
+                assert np.array_equal(g[special], rounded[special], equal_nan=True), k
+                assert np.all(np.abs(g[~special] - want[~special]) <= SUM_REL * mag[~special]), k
+                sq = np.float32((x.astype(np.float64) ** 2).sum())
+                assert np.array_equal(sums[k], sq, equal_nan=True) if not np.isfinite(sq) else abs(sums[k] - sq) <= SUM_REL * sq, k
+
+
+@pytest.mark.parametrize("shape", [s for s in SHAPES if len(s) == 1], ids=str)
+@pytest.mark.parametrize("pattern", PATTERNS)
+def test_noalloc(shape, pattern):
+    import torch
+    sk = skel()
+    x = sequence(shape, pattern)
+    out = dev_empty(shape, torch.float32)
+    for inclusive in (True, False):
+        sk.skel_scan_noalloc("add", inclusive, dev_tensor(x), out)
+        got, (want, mag) = to_np(out), prefixes(x, inclusive, False)
+        with np.errstate(all="ignore"):
+            rounded = want.astype(np.float32)
+            special = ~np.isfinite(rounded)
+            assert np.array_equal(got[special], rounded[special], equal_nan=True)
+            assert np.all(np.abs(got[~special] - want[~special]) <= SUM_REL * mag[~special])
