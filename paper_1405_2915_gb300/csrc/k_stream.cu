@@ -189,24 +189,36 @@ st2_stream(const float *__restrict__ in, float *__restrict__ out, int64_t rows, 
                     const bool up = ROWE && top && i == 0, down = ROWE && bottom && i == nin - 1;
 #pragma unroll
                     for (int j = 0; j < C; ++j) {
-                        if (up) P2[0][j] = fmaf(w.w[8], e[j + 2], fmaf(w.w[7], e[j + 1], fmaf(w.w[6], e[j], P2[0][j])));
-                        if (down) P2[0][j] = fmaf(w.w[2], e[j + 2], fmaf(w.w[1], e[j + 1], fmaf(w.w[0], e[j], P2[0][j])));
+                        if (up) {
+                            if (!TAPS5) P2[0][j] = fmaf(w.w[6], e[j], P2[0][j]);
+                            P2[0][j] = fmaf(w.w[7], e[j + 1], P2[0][j]);
+                            if (!TAPS5) P2[0][j] = fmaf(w.w[8], e[j + 2], P2[0][j]);
+                        }
+                        if (down) {
+                            if (!TAPS5) P2[0][j] = fmaf(w.w[0], e[j], P2[0][j]);
+                            P2[0][j] = fmaf(w.w[1], e[j + 1], P2[0][j]);
+                            if (!TAPS5) P2[0][j] = fmaf(w.w[2], e[j + 2], P2[0][j]);
+                        }
                         if (!COLE) continue;
                         // likewise the columns beside the grid: one tap per row of the first, of the last column
                         const float v = e[j + 1];
                         if (lead && j == 0) {
-                            x[j] = fmaf(w.w[8], v, x[j]);
                             P2[0][j] = fmaf(w.w[5], v, P2[0][j]);
-                            P1[0][j] = fmaf(w.w[2], v, P1[0][j]);
-                            if (up) P2[0][j] = fmaf(w.w[8], v, P2[0][j]);
-                            if (down) P2[0][j] = fmaf(w.w[2], v, P2[0][j]);
+                            if (!TAPS5) {
+                                x[j] = fmaf(w.w[8], v, x[j]);
+                                P1[0][j] = fmaf(w.w[2], v, P1[0][j]);
+                                if (up) P2[0][j] = fmaf(w.w[8], v, P2[0][j]);
+                                if (down) P2[0][j] = fmaf(w.w[2], v, P2[0][j]);
+                            }
                         }
                         if (trail && j == nv - 1) {
-                            x[j] = fmaf(w.w[6], v, x[j]);
                             P2[0][j] = fmaf(w.w[3], v, P2[0][j]);
-                            P1[0][j] = fmaf(w.w[0], v, P1[0][j]);
-                            if (up) P2[0][j] = fmaf(w.w[6], v, P2[0][j]);
-                            if (down) P2[0][j] = fmaf(w.w[0], v, P2[0][j]);
+                            if (!TAPS5) {
+                                x[j] = fmaf(w.w[6], v, x[j]);
+                                P1[0][j] = fmaf(w.w[0], v, P1[0][j]);
+                                if (up) P2[0][j] = fmaf(w.w[6], v, P2[0][j]);
+                                if (down) P2[0][j] = fmaf(w.w[0], v, P2[0][j]);
+                            }
                         }
                     }
                 }
