@@ -25,6 +25,7 @@ namespace {
 // written once.  Progress, bounded waits and the ticket reset as in scan
 // variant 8.
 constexpr int kBrTE = 4096;    // elements per tile
+constexpr int kBrChunk = 128;  // tiles of an instance that are placed by a warp of their own
 constexpr int kBrAggW = 2;     // aggregator warps
 constexpr int kBrQueue = 16;   // queue entries per block
 constexpr int kBrOffCap = 64;  // instance offsets a scanner keeps per tile (more: searched in global memory)
@@ -68,11 +69,33 @@ struct BrFF : dev::Sum2 {
     __device__ __forceinline__ void set(double v) { *static_cast<dev::Sum2 *>(this) = dev::Sum2(v); }
 };
 
-// Checks the offsets and writes each tile's placement, one warp per instance:
-// the tiles whose first element it holds get its number, the tiles whose last
-// element it holds its start.  No searches: two dependent loads, then stores
-// (a search per tile was twelve dependent loads, and the check a kernel of
-// one block: 5.4 + 7.7 us for 4096 instances, now 3.3 in one launch).
+// The instance holding element v: the largest b in [0, B) with off[b] <= v
+// (sorted offsets; off[0] = 0 <= v < off[B]).  One warp, 32 probes a round.
+__device__ __forceinline__ int64_t br_instance_of(const int64_t *__restrict__ off, int64_t B, int64_t v)
+{
+    const int lane = threadIdx.x & 31;
+    int64_t a = 0, n = B;   // it is one of a .. a + n - 1
+    while (n > 1) {
+        const int64_t step = (n + 31) / 32, p = a + (lane + 1) * step;
+        const int below = __popc(__ballot_sync(0xffffffffu, p < a + n && __ldg(off + p) <= v));
+        a += below * step;
+        n = step < n - below * step ? step : n - below * step;
+    }
+    return a;
+}
+
+// Checks the offsets and writes each tile's placement: the tiles whose first
+// element an instance holds get its number, the tiles whose last element it
+// holds its start.  One warp per instance, or where there are more instances
+// than warps one lane, which leaves those of several tiles to the warp.  No
+// searches: two dependent loads, then stores (a search per tile was twelve
+// dependent loads, and the check a kernel of one block: 5.4 + 7.7 us for 4096
+// instances, now 3.3 in one launch).  A long instance has more tiles than a
+// warp should write (65536 for 2^28 elements), so every run of kBrChunk tiles
+// that lies in one instance is left to a warp of its own, which finds the
+// instance by a search (whole calls, us, one warp per instance -> now: one
+// instance of 2^28 718 -> 569, 2^27 and 4095 of 100 396 -> 322, a million of
+// 300 T1).
 // Invalid offsets are reported and, unless `alone` (no main kernel follows),
 // make the main kernel return at once; the placements they give are only
 // kept inside the array.
@@ -81,27 +104,60 @@ batched_br_place(const int64_t *__restrict__ off, int64_t B, int64_t total, floa
                  BrMeta *__restrict__ meta, Control *ctl, int alone)
 {
     dev::grid_wait();
+    constexpr int64_t CE = (int64_t)kBrChunk * kBrTE;
     const int lane = threadIdx.x & 31;
-    const int64_t ntiles = (total + kBrTE - 1) / kBrTE;
+    const int64_t ntiles = (total + kBrTE - 1) / kBrTE, nchunks = total / CE, warps = (int64_t)gridDim.x * 8;
+    const int group = B > warps ? 32 : 1;   // instances per warp and round
     bool bad = blockIdx.x == 0 && threadIdx.x == 0 && (off[0] != 0 || off[B] != total);
-    for (int64_t b = (int64_t)blockIdx.x * 8 + (threadIdx.x >> 5); b < B; b += (int64_t)gridDim.x * 8) {
-        const int64_t lo = __ldg(off + b), hi = __ldg(off + b + 1);
-        if (hi <= lo) {
-            bad |= hi < lo;
-            if (lane == 0 && hi == lo && results) results[b] = 0.f;
+    for (int64_t k = (int64_t)blockIdx.x * 8 + (threadIdx.x >> 5); k < nchunks + (B + group - 1) / group; k += warps) {
+        if (k < nchunks) {
+            const int64_t b = br_instance_of(off, B, k * CE), lo = __ldg(off + b), hi = __ldg(off + b + 1);
+            if (lo <= k * CE && hi >= (k + 1) * CE)
+                for (int i = lane; i < kBrChunk; i += 32) meta[k * kBrChunk + i] = BrMeta{b, lo};
             continue;
         }
-        if (lo < 0 || hi > total) {
-            bad = true;
-            continue;
+        // tiles [f0, f1) start in the lane's instance [lo, hi), tiles [l0, l1) end in it
+        const int64_t first = (k - nchunks) * group, b = first + lane;
+        int64_t lo = 0, hi = 0, f0 = 0, f1 = 0, l0 = 0, l1 = 0;
+        if (lane < group && b < B) {
+            lo = __ldg(off + b);
+            hi = __ldg(off + b + 1);
+            if (hi == lo) {
+                if (results) results[b] = 0.f;
+            } else if (hi < lo || lo < 0 || hi > total) {
+                bad = true;
+            } else {
+                const uint64_t ulo = (uint64_t)lo, uhi = (uint64_t)hi;   // shifts, not signed divisions
+                f0 = (ulo + kBrTE - 1) / kBrTE;
+                f1 = (uhi + kBrTE - 1) / kBrTE;
+                l0 = ulo / kBrTE;
+                l1 = hi == total ? ntiles : uhi / kBrTE;
+            }
         }
-        // first elements t * TE in [lo, hi)
-        for (int64_t t = (lo + kBrTE - 1) / kBrTE + lane; t * kBrTE < hi; t += 32) meta[t].b0 = b;
-        // last elements (t + 1) * TE - 1, of the last tile total - 1, in [lo, hi)
-        for (int64_t t = lo / kBrTE + lane; t < ntiles; t += 32) {
-            const int64_t last = (t + 1) * kBrTE < total ? (t + 1) * kBrTE - 1 : total - 1;
-            if (last >= hi) break;
-            meta[t].hp = lo;
+        const bool few = f1 - f0 <= 1 && l1 - l0 <= 1;
+        if (few) {
+            if (f0 < f1) meta[f0].b0 = b;
+            if (l0 < l1) meta[l0].hp = lo;
+        }
+        for (uint32_t left = __ballot_sync(0xffffffffu, !few); left; left &= left - 1) {
+            const int src = __ffs(left) - 1;
+            const int64_t wlo = __shfl_sync(0xffffffffu, lo, src), whi = __shfl_sync(0xffffffffu, hi, src);
+            const int64_t wf0 = __shfl_sync(0xffffffffu, f0, src), wf1 = __shfl_sync(0xffffffffu, f1, src);
+            const int64_t wl0 = __shfl_sync(0xffffffffu, l0, src), wl1 = __shfl_sync(0xffffffffu, l1, src);
+            int64_t s0 = wf1, s1 = wf1;   // the whole runs [s0, s1) are left out (l1 <= f1)
+            if (wf1 - wf0 >= kBrChunk) {
+                const int64_t c0 = (wlo + CE - 1) / CE, c1 = whi / CE;
+                if (c0 < c1) {
+                    s0 = c0 * kBrChunk;
+                    s1 = c1 * kBrChunk;
+                }
+            }
+            for (int64_t t = wf0 + lane; t < s0; t += 32) meta[t].b0 = first + src;
+            for (int64_t t = wl0 + lane; t < wl1 && t < s0; t += 32) meta[t].hp = wlo;
+            if (s1 < wf1) {
+                for (int64_t t = s1 + lane; t < wf1; t += 32) meta[t].b0 = first + src;
+                for (int64_t t = s1 + lane; t < wl1; t += 32) meta[t].hp = wlo;
+            }
         }
     }
     if (bad) {
@@ -583,7 +639,7 @@ int run_br(const BatchedLaunch &b, const Choice &c, Control *ctl, uint64_t *word
     const int64_t ntiles = ceil_div(b.total, (int64_t)kBrTE);
     if (ntiles > 0x7fffffffLL) return fail(SKEL_ERR_SHAPE, "batched: too many tiles");
     BrMeta *meta = reinterpret_cast<BrMeta *>(data + 256);
-    const int64_t pgrid = std::max<int64_t>(1, std::min<int64_t>(ceil_div(b.B, (int64_t)8), (int64_t)device_info().sms * 8));
+    const int64_t pgrid = std::max<int64_t>(1, std::min<int64_t>(ceil_div(b.B + ntiles / kBrChunk, (int64_t)8), (int64_t)device_info().sms * 8));
     launch_kernel(batched_br_place, (unsigned)pgrid, 256, 0, s, b.offsets, b.B, b.total, b.results, meta, ctl,
                   b.total == 0 ? 1 : 0);
     cudaError_t e = cudaPeekAtLastError();

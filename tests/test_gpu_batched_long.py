@@ -1,0 +1,55 @@
+"""Batched variant 7 with instances of several hundred tiles (their placement is
+split over warps): starts and ends on, before and after the boundary of a run
+of 128 tiles of 4096 elements, alone, among short ones and among empty ones."""
+import numpy as np
+import pytest
+
+from helpers import forced, skel, wrap
+
+pytestmark = pytest.mark.gpu
+
+RUN = 128 * 4096
+CASES = {
+    "one": [5 * RUN + 17],
+    "one_run": [RUN],
+    "short_of_a_run": [RUN - 1],
+    "past_a_run": [RUN + 1],
+    "runs": [RUN, 2 * RUN, RUN],
+    "between_short": [100] * 50 + [3 * RUN] + [100] * 50,
+    "shifted": [1, 2 * RUN - 1, 3 * RUN + 1, 4095, 2 * RUN],
+    "empty_around": [0, 0, 2 * RUN, 0, 0, 0, 2 * RUN + 5, 0],
+    "many": [7] * 3000 + [4 * RUN + 3] + [4096] * 40 + [2 * RUN],
+    "more_than_warps": [300] * 20_000 + [0, RUN + 3, 9000] + [4096, 8192, 1, 0] * 5_000 + [2 * RUN, 5],
+    "ends_in_a_part_tile": [RUN, RUN - 4096 + 1],
+}
+
+
+@pytest.mark.parametrize("case", CASES)
+def test_long_instances(case):
+    import torch
+    sk = skel()
+    lens = CASES[case]
+    off = np.concatenate([[0], np.cumsum(lens)]).astype(np.int64)
+    n = int(off[-1])
+    # whole numbers: every order of the sums is exact in float32
+    v = torch.randint(0, 2, (n,), device="cuda", dtype=torch.int32).float()
+    do = torch.from_numpy(off).cuda()
+    res, out = torch.full((len(lens),), -1.0, device="cuda"), torch.full((n,), -1.0, device="cuda")
+    s = v.double().cumsum(0)
+    before = torch.cat([s.new_zeros(1), s])[do]                       # the sum before each instance's first element
+    start = torch.repeat_interleave(before[:-1], do[1:] - do[:-1])
+    for inclusive in (True, False):
+        with forced("batched", 7, 0, 4, 0):
+            sk.skel_batched(wrap(v), wrap(do), wrap(res), wrap(out), inclusive)
+        sk.skel_check_device()
+        assert torch.equal(res.double(), before[1:] - before[:-1])
+        assert torch.equal(out.double(), s - start - (0 if inclusive else v.double()))
+    # unsorted offsets are still rejected (instances that the bad offsets make empty may be written)
+    bad = do.clone()
+    bad[0] = n
+    res.fill_(7.0)
+    with forced("batched", 7, 0, 4, 0):
+        sk.skel_batched(wrap(v), wrap(bad), wrap(res), wrap(out), True)
+    with pytest.raises(sk.SkelError):
+        sk.skel_check_device()
+    assert bool((res[bad[1:] != bad[:-1]] == 7.0).all())
