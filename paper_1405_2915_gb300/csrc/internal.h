@@ -83,7 +83,7 @@ struct Control {
     uint32_t queue;      // work queue of persistent kernels
     uint32_t exited;     // persistent blocks that left the work loop
     uint32_t epoch;      // last look-back tag of a kernel that keeps its tag on the device (0: none yet)
-    uint32_t reject;     // a call's device-resident input failed validation (reset by that call's last kernel)
+    uint32_t reject;     // epoch of a call whose device-resident input failed validation; its main kernel returns
     uint32_t pad[56];
 };
 static_assert(sizeof(Control) == 256, "control block is 256 bytes");

@@ -760,10 +760,11 @@ Choice batched_default() { return Choice{5, 256, 8, 0}; }
 
 size_t batched_data_bytes(const BatchedLaunch &b, const Choice &c)
 {
-    // the flat variants: a flag and, per tile, its first instance (6) or a
-    // 16-byte placement (7)
-    if (c.variant == 6 || c.variant == 7)
-        return 256 + (c.variant == 6 ? 8 : 16) * (size_t)ceil_div(b.total, (int64_t)tile_of(c));
+    // the flat variants: per tile a 16-byte placement (7), or its first
+    // instance, after a flag (6)
+    const size_t flat_tiles = (size_t)ceil_div(b.total, (int64_t)tile_of(c));
+    if (c.variant == 7) return 16 * flat_tiles;
+    if (c.variant == 6) return 256 + 8 * flat_tiles;
     // reduce-then-scan also keeps three float64 values per tile and, from the
     // next 256-byte boundary, a 32-byte placement per tile
     if (c.variant != 5) return layout_bytes(b, tile_of(c));

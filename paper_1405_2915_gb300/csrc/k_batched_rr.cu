@@ -95,13 +95,14 @@ __device__ __forceinline__ int64_t br_instance_of(const int64_t *__restrict__ of
 // that lies in one instance is left to a warp of its own, which finds the
 // instance by a search (whole calls, us, one warp per instance -> now: one
 // instance of 2^28 718 -> 569, 2^27 and 4095 of 100 396 -> 322, a million of
-// 300 T1).
+// 300 1461 -> 1385; by a search per tile 580, 335 and 1785).
 // Invalid offsets are reported and, unless `alone` (no main kernel follows),
-// make the main kernel return at once; the placements they give are only
-// kept inside the array.
+// make the call's main kernel return at once, by the call's tag: should that
+// launch fail, no later call takes the flag for its own.  The placements that
+// invalid offsets give are only kept inside the array.
 __global__ void __launch_bounds__(256)
 batched_br_place(const int64_t *__restrict__ off, int64_t B, int64_t total, float *__restrict__ results,
-                 BrMeta *__restrict__ meta, Control *ctl, int alone)
+                 BrMeta *__restrict__ meta, Control *ctl, uint32_t epoch, int alone)
 {
     dev::grid_wait();
     constexpr int64_t CE = (int64_t)kBrChunk * kBrTE;
@@ -162,7 +163,7 @@ batched_br_place(const int64_t *__restrict__ off, int64_t B, int64_t total, floa
     }
     if (bad) {
         atomicOr(&ctl->error, kErrInput);
-        if (!alone) atomicExch(&ctl->reject, 1u);
+        if (!alone) atomicExch(&ctl->reject, epoch);
     }
 }
 
@@ -188,7 +189,7 @@ batched_br(const float *__restrict__ values, const int64_t *__restrict__ off, in
     __shared__ int q_tail, q_claim, q_read, a_done, s_stop;
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
     const int64_t ntiles = (total + TE - 1) / TE, nfull = total / TE;
-    if (dev::ld_volatile(&ctl->reject)) {   // invalid offsets (reported): every block leaves, no ticket drawn
+    if (dev::ld_volatile(&ctl->reject) == epoch) {   // invalid offsets (reported): every block leaves, no ticket drawn
         __syncthreads();                    // every thread has read the flag
         if (threadIdx.x == 0 && atomicAdd(&ctl->exited, 1u) == gridDim.x - 1) {   // ... and every block
             ctl->reject = 0u;
@@ -602,24 +603,35 @@ batched_br(const float *__restrict__ values, const int64_t *__restrict__ off, in
     }
 }
 
+int run_br_place(const BatchedLaunch &b, Control *ctl, BrMeta *meta, uint32_t epoch, bool alone, cudaStream_t s)
+{
+    const int64_t warps = b.B + b.total / ((int64_t)kBrChunk * kBrTE), most = (int64_t)device_info().sms * 8;
+    const int64_t grid = std::max<int64_t>(1, std::min<int64_t>(ceil_div(warps, (int64_t)8), most));
+    launch_kernel(batched_br_place, (unsigned)grid, 256, 0, s, b.offsets, b.B, b.total, b.results, meta, ctl, epoch, (int)alone);
+    const cudaError_t e = cudaPeekAtLastError();
+    return e == cudaSuccess ? SKEL_OK : fail_cuda(cudaGetLastError(), "batched reread placement launch");
+}
+
 template <bool SCAN, bool RED, bool INCL, int R, int NC>
-int run_br_k(const BatchedLaunch &b, Control *ctl, uint64_t *words, const BrMeta *meta, uint32_t epoch, cudaStream_t s)
+int run_br_k(const BatchedLaunch &b, Control *ctl, uint64_t *words, BrMeta *meta, uint32_t epoch, cudaStream_t s)
 {
     auto kern = batched_br<SCAN, RED, INCL, R, NC>;
     const int dyn = (R + NC) * kBrTE * 4, threads = (kBrAggW + NC) * 32;
     const int occ = kernel_occupancy(kern, threads, dyn);
     if (occ < 1) return fail(SKEL_ERR_UNSUPPORTED, "batched reread: kernel does not fit an SM");
+    const int rc = run_br_place(b, ctl, meta, epoch, false, s);
+    if (rc) return rc;
     const int64_t ntiles = ceil_div(b.total, (int64_t)kBrTE);
     dev::LookbackDesc d{words, words + 2 * ntiles};
     const DebugKnobs k = debug_knobs();
     launch_kernel(kern, (unsigned)(device_info().sms * occ), threads, (size_t)dyn, s, b.values, b.offsets, b.B,
-                  b.total, b.results, b.scan_out, meta, d, ctl, epoch, k.scan_skip_publish_tile, k.wait_limit_ns);
+                  b.total, b.results, b.scan_out, (const BrMeta *)meta, d, ctl, epoch, k.scan_skip_publish_tile, k.wait_limit_ns);
     const cudaError_t e = cudaPeekAtLastError();
     return e == cudaSuccess ? SKEL_OK : fail_cuda(cudaGetLastError(), "batched reread launch");
 }
 
 template <int R, int NC>
-int run_br_shape(const BatchedLaunch &b, Control *ctl, uint64_t *words, const BrMeta *meta, uint32_t epoch, cudaStream_t s)
+int run_br_shape(const BatchedLaunch &b, Control *ctl, uint64_t *words, BrMeta *meta, uint32_t epoch, cudaStream_t s)
 {
     if (b.want_scan && b.want_reduce)
         return b.inclusive ? run_br_k<true, true, true, R, NC>(b, ctl, words, meta, epoch, s)
@@ -638,13 +650,8 @@ int run_br(const BatchedLaunch &b, const Choice &c, Control *ctl, uint64_t *word
     if (c.tile < 0 || c.tile > 1) return fail(SKEL_ERR_INVALID_ARG, "batched reread: tile must be 0 or 1");
     const int64_t ntiles = ceil_div(b.total, (int64_t)kBrTE);
     if (ntiles > 0x7fffffffLL) return fail(SKEL_ERR_SHAPE, "batched: too many tiles");
-    BrMeta *meta = reinterpret_cast<BrMeta *>(data + 256);
-    const int64_t pgrid = std::max<int64_t>(1, std::min<int64_t>(ceil_div(b.B + ntiles / kBrChunk, (int64_t)8), (int64_t)device_info().sms * 8));
-    launch_kernel(batched_br_place, (unsigned)pgrid, 256, 0, s, b.offsets, b.B, b.total, b.results, meta, ctl,
-                  b.total == 0 ? 1 : 0);
-    cudaError_t e = cudaPeekAtLastError();
-    if (e != cudaSuccess) return fail_cuda(cudaGetLastError(), "batched reread prep launch");
-    if (b.total == 0) return SKEL_OK;
+    BrMeta *meta = reinterpret_cast<BrMeta *>(data);
+    if (b.total == 0) return run_br_place(b, ctl, meta, epoch, true, s);
     return c.tile ? run_br_shape<4, 8>(b, ctl, words, meta, epoch, s)
                   : run_br_shape<6, 6>(b, ctl, words, meta, epoch, s);
 }

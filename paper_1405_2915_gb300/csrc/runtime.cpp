@@ -179,6 +179,14 @@ std::vector<GraphBlock *> &graph_blocks()
 
 size_t round256(size_t b) { return (b + 255) & ~(size_t)255; }
 
+// Everything that holds a call's tag: the control words from `abort` on (the
+// counters among them are 0 between calls) and the look-back words behind them.
+cudaError_t clear_tags(unsigned char *base, size_t words, cudaStream_t stream)
+{
+    const size_t skip = offsetof(Control, abort);
+    return cudaMemsetAsync(base + skip, 0, sizeof(Control) - skip + words * 8, stream);
+}
+
 // Whether `stream` is being captured, and into which graph.
 bool capture_of(cudaStream_t stream, unsigned long long *id, cudaGraph_t *graph)
 {
@@ -275,9 +283,8 @@ int capture_scratch(int dev, cudaStream_t stream, unsigned long long id, cudaGra
     out->data = base + sizeof(Control) + b->word_cap * 8;
     out->data_bytes = b->data_cap;
     out->epoch = 1;
-    if (word_count > 0) {   // one node: the control words from `abort` on, and the look-back words behind them
-        const size_t skip = offsetof(Control, abort);
-        cudaError_t e = cudaMemsetAsync(base + skip, 0, sizeof(Control) - skip + word_count * 8, stream);
+    if (word_count > 0) {   // a node of the graph
+        cudaError_t e = clear_tags(base, word_count, stream);
         if (e != cudaSuccess) return fail_cuda(e, "look-back word clear");
     }
     return SKEL_OK;
@@ -325,10 +332,9 @@ int get_scratch(cudaStream_t stream, size_t data_bytes, size_t word_count, Scrat
     out->data_bytes = b.data_cap;
     if (word_count > 0) {
         b.epoch += 1;
-        if (b.epoch > kMaxEpoch) {   // tag space used up: clear every word and the abort tag, restart
+        if (b.epoch > kMaxEpoch) {   // tag space used up: clear every word and the calls' tags, restart
             b.epoch = 1;
-            cudaError_t e = cudaMemsetAsync(out->words, 0, b.word_cap * 8, stream);
-            if (e == cudaSuccess) e = cudaMemsetAsync(&out->ctl->abort, 0, sizeof(uint32_t), stream);
+            cudaError_t e = clear_tags(base, b.word_cap, stream);
             if (e != cudaSuccess) return fail_cuda(e, "look-back word clear");
         }
     }

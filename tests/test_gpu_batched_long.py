@@ -53,3 +53,42 @@ def test_long_instances(case):
     with pytest.raises(sk.SkelError):
         sk.skel_check_device()
     assert bool((res[bad[1:] != bad[:-1]] == 7.0).all())
+
+
+def test_a_stale_rejection_flag_is_not_the_next_calls():
+    """A call whose placement rejected its offsets and whose main kernel never
+    ran leaves its tag in the scratch's control block; later calls run, past the
+    wrap of the tags too."""
+    import torch
+    sk = skel()
+    s, blocks = torch.cuda.Stream(), []
+
+    def alloc(size, stream, ctx):
+        blocks.append(torch.zeros(int(size) + 256, dtype=torch.uint8, device="cuda"))
+        return (blocks[-1].data_ptr() + 255) // 256 * 256
+
+    a, f = sk._lib.ALLOC_FN(alloc), sk._lib.FREE_FN(lambda p, stream, ctx: None)
+    lens = [3000, 5000, 1, 9000]
+    off = torch.from_numpy(np.concatenate([[0], np.cumsum(lens)]).astype(np.int64)).cuda()
+    v = torch.ones(int(off[-1]), device="cuda")
+    res, want = torch.empty(4, device="cuda"), torch.tensor(lens, device="cuda", dtype=torch.float32)
+    c = [wrap(v), wrap(off), wrap(res), None]
+    torch.cuda.synchronize()
+    sk.check(sk.lib.skel_set_allocator(a, f, None))
+    try:
+        with forced("batched", 7, 0, 4, 0):
+            sk.skel_batched(*c, True, stream=s)                 # the call's tag is 1
+            s.synchronize()
+            assert len(blocks) == 1                             # the stream's scratch
+            flag = blocks[0][(-blocks[0].data_ptr()) % 256:][28:32].view(torch.int32)
+            flag.fill_(1)                                       # as the failed call would leave it
+            for k in range(260):
+                res.zero_()
+                torch.cuda.synchronize()
+                sk.skel_batched(*c, True, stream=s)
+                s.synchronize()
+                assert torch.equal(res, want), k
+            sk.skel_check_device(s)
+    finally:
+        sk.check(sk.lib.skel_release_cached())
+        sk.use_torch_allocator(False)
