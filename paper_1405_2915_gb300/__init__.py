@@ -231,10 +231,15 @@ class Container:
 _HANDLES = [C.c_void_p * k for k in range(4)]
 
 
+def _closed():
+    raise SkelError(_lib.ERR_INVALID_ARG, "container is closed")
+
+
 def _handles(cs: Sequence[Container | None]):
     n = len(cs)
     arr = _HANDLES[n] if 0 < n < 4 else C.c_void_p * max(1, n)
-    return arr(*[None if c is None else c._h for c in cs])
+    # a closed container is an error, not an operand that is not wanted
+    return arr(*[None if c is None else c._h or _closed() for c in cs])
 
 
 def _fn(name) -> int:
