@@ -24,7 +24,7 @@
 // planes (plane p holds the p-th group of four columns of every thread, so
 // 16-byte reads are free of bank conflicts) and out by contiguous stores.
 //
-// What bounds it (8192 x 8192): the forward takes 127 us, the backward 176
+// What bounds it (8192 x 8192): the forward takes 127 us, the backward 174
 // (180 and 235 with cp.async), against 79 us each for their HBM traffic
 // (which ncu shows at 1.0 of the algorithmic bytes): instruction issue, active
 // 71 and 61 % of the time, with 16 warps per SM whose barriers keep them in the
@@ -33,13 +33,22 @@
 // therefore splits its barrier into an arrival and a wait, with the stencil's
 // inner columns and the next row's tanh between them (136 us with one whole
 // barrier; the backward, at 128 registers, spills when split so: 209).  As
-// fifteen separate calls the loss and its gradient took 927 us, here 304.  512
+// fifteen separate calls the loss and its gradient took 927 us, here 301.  512
 // threads of 16 columns: with 1024 of 8 the scans' shuffles and the edges
 // weigh twice as much.
 //
-// Sums run per thread with their rounding errors kept, then in float64 over
-// threads and blocks; the last block to finish adds the blocks' partial sums
-// in index order (deterministic) and writes L.
+// The two sums of squares run per thread with their rounding errors kept, then
+// in float64 over threads and blocks; the last block to finish adds the
+// blocks' partial sums in index order (deterministic) and writes L.
+//
+// Row prefixes are float32: a value passes at most 17 roundings (6 in its
+// thread, 5 in its warp, 4 between warps, 2 to put them together), so the
+// error of s is at most 17 2^-24 of the prefix of |t|.  The reverse scan keeps
+// the rounding errors between warps, where its sums are the largest, as its
+// error reaches gx directly.  Relative error of gx (norm) on rows of one sign,
+// U[0, 0.02], plain -> kept, and separate calls whose scans carry float64
+// between tiles of 4096: 2048 x 8191 5.9e-8 -> 5.4e-8, 5.6e-8; 64 x 8192 7.3e-8
+// -> 6.3e-8, 7.7e-8.
 #include <type_traits>
 
 #include "stencil.cuh"
@@ -118,12 +127,6 @@ __device__ __forceinline__ float scan_thread(float (&v)[C])
     return off;
 }
 
-__device__ __forceinline__ float warp_sum(float v)
-{
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-    return v;
-}
 __device__ __forceinline__ double warp_sum(double v)
 {
 #pragma unroll
@@ -420,12 +423,38 @@ __device__ __forceinline__ float warp_exclusive(float wi, int lane)
     return lane == (REV ? 31 : 0) ? 0.f : q;
 }
 
-// Sum of the totals of the warps before (REV: after) `warp`.
+// Sum of the totals of the warps before (REV: after) `warp`: each half-warp
+// adds them up in a tree.
+constexpr int kOffsetLanes = 16;
+static_assert(kLMaxCols / kFwdC <= 32 * kOffsetLanes && kLMaxCols / kBwdC <= 32 * kOffsetLanes, "a lane per warp");
+template <bool REV>
+__device__ __forceinline__ float lane_total(const Exchange &ex, int lane, int warp, int nwarps)
+{
+    const int k = lane & (kOffsetLanes - 1);
+    return (REV ? k > warp && k < nwarps : k < warp) ? ex.total[k] : 0.f;
+}
 template <bool REV>
 __device__ __forceinline__ float warp_offset(const Exchange &ex, int lane, int warp, int nwarps)
 {
-    const bool in = REV ? lane > warp && lane < nwarps : lane < warp;
-    return warp_sum(in ? ex.total[lane] : 0.f);
+    float v = lane_total<REV>(ex, lane, warp, nwarps);
+#pragma unroll
+    for (int o = kOffsetLanes / 2; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+    return v;
+}
+// The same with its rounding errors kept.
+template <bool REV>
+__device__ __forceinline__ dev::Sum2 warp_offset2(const Exchange &ex, int lane, int warp, int nwarps)
+{
+    dev::Sum2 r;
+    r.hi = lane_total<REV>(ex, lane, warp, nwarps);
+    r.add(__shfl_xor_sync(0xffffffffu, r.hi, kOffsetLanes / 2));
+#pragma unroll
+    for (int o = kOffsetLanes / 4; o > 0; o >>= 1) {
+        const float h = __shfl_xor_sync(0xffffffffu, r.hi, o), l = __shfl_xor_sync(0xffffffffu, r.lo, o);
+        r.add(h);
+        r.lo += l;
+    }
+    return r;
 }
 
 // ------------------------------------------------------------- forward --
@@ -575,6 +604,8 @@ loss_bwd(const __grid_constant__ CUtensorMap tin, const __grid_constant__ CUtens
     const int64_t q0 = r0 > 2 ? r0 - 2 : 0;
     const bool clamp = b == SKEL_CLAMP;
     const int nin = (int)((r1 + 2 < rows ? r1 + 2 : rows) - q0), niter = (int)(r1 + 2 - q0);
+    // the iterations of rows 1, `rows` (past them if it is not reached) and r0 + 2
+    const int i1 = q0 > 1 ? -1 : (int)(1 - q0), ilast = rows - q0 < niter ? (int)(rows - q0) : niter, iout = (int)(r0 + 2 - q0);
     RowStream<MODE, C, kBwdRing> rs(t, rows, cols, q0, nin, dyn, &tin, &tout, ctl);
     const int lane = rs.lane, warp = rs.warp;
     const float g2 = 2.f * __ldg(g), gc2 = 2.f * ((float)(1.0 / ((double)rows * (double)cols)) * __ldg(g));
@@ -591,8 +622,7 @@ loss_bwd(const __grid_constant__ CUtensorMap tin, const __grid_constant__ CUtens
     __syncthreads();
 
     for (int i = 0; i < niter; ++i) {
-        const int64_t row = q0 + i;
-        const bool out_row = row - 2 >= r0;   // (row - 2 < r1 by the loop's bound)
+        const bool out_row = i >= iout;       // row q0 + i - 2 is one of the block's (below r1 by the loop's bound)
         // ---- phase 1: the arriving row, the scan of row - 2 ----
         float v[C];
         if (i < nin) rs.await(i);
@@ -626,9 +656,9 @@ loss_bwd(const __grid_constant__ CUtensorMap tin, const __grid_constant__ CUtens
                 if (rs.trail && j == rs.nv) e[j + 1] = clamp ? v[j - 1] : 0.f;
         }
         float u[C];
-        if (row == 0 && clamp) add_row_above<ROW_ALL>(w, e, P1);
+        if (i == i1 - 1 && clamp) add_row_above<ROW_ALL>(w, e, P1);
         add_row<ROW_ALL>(w, W3{{w.w[3], w.w[4], w.w[5]}}, e, P1, P2, u);
-        if (row >= 1 && row <= rows) {                     // row - 1 is a row of the grid
+        if (i >= i1 && i <= ilast) {                       // the row above is a row of the grid
 #pragma unroll
             for (int j = 0; j < C; ++j) u[j] *= g2;
             rs.mask(u);
@@ -658,6 +688,11 @@ loss_bwd(const __grid_constant__ CUtensorMap tin, const __grid_constant__ CUtens
         __syncthreads();
         if (MODE == kTma) rs.template copy_next<0>();   // here: the slot's store has had this row's two phases to end
         // ---- phase 3: the adjoint stencil of row - 2, gx of row - 2 ----
+        float back = 0.f;                     // the reverse scan's offset; formed before the stencil: both passes 301 us, after it 306
+        if (out_row) {
+            const dev::Sum2 off = warp_offset2<true>(ex[1], lane, warp, rs.nwarps);
+            back = off.hi + (off.low() + warp_exclusive<true>(rwi, lane));
+        }
         neighbours(u, lane, e);               // 0 outside the grid
         warp_neighbours<C>(ex[1], lane, warp, rs.nwarps, e);
         // CLAMP: taps that the forward clamped onto the grid's edge.  The
@@ -667,11 +702,11 @@ loss_bwd(const __grid_constant__ CUtensorMap tin, const __grid_constant__ CUtens
         // (one tap per row of the first, and of the last, column) is summed
         // apart and added to the edge column.
         W3 m{{wt.w[3], wt.w[4], wt.w[5]}};
-        if (clamp && row == 1) {
+        if (clamp && i == i1) {
 #pragma unroll
             for (int k = 0; k < 3; ++k) m.w[k] += wt.w[6 + k];
         }
-        if (clamp && row == rows) {
+        if (clamp && i == ilast) {
 #pragma unroll
             for (int k = 0; k < 3; ++k) m.w[k] += wt.w[k];
         }
@@ -691,12 +726,11 @@ loss_bwd(const __grid_constant__ CUtensorMap tin, const __grid_constant__ CUtens
             for (int j = 0; j < C; ++j) gt[j] += rs.trail && j == rs.nv - 1 ? orr : 0.f;
         }
         if (out_row) {
-            const float base = warp_offset<true>(ex[1], lane, warp, rs.nwarps) + warp_exclusive<true>(rwi, lane);
             float y[C];
             rs.read(i - 2, y);
 #pragma unroll
-            for (int j = 0; j < C; ++j) y[j] = (gt[j] + (sc[j] + base)) * fmaf(-y[j], y[j], 1.f);
-            rs.write(i - 2, y, gx, row - 2);
+            for (int j = 0; j < C; ++j) y[j] = (gt[j] + (sc[j] + back)) * fmaf(-y[j], y[j], 1.f);
+            rs.write(i - 2, y, gx, q0 + i - 2);
         }
         rs.end_stores();
     }
