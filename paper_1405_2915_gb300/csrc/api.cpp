@@ -527,14 +527,21 @@ struct ScalarResult {
 
 Choice scan_def();
 
-// A scan's variant.  The table is keyed by the total size alone; two rules
-// add what it cannot see.  Rows: one block per row (variant 9) wherever a row
-// fits a block's shared memory and either there is a row for every second SM
-// or a row is short (4097 x 4099 38 us against 298, 8192 x 256 9 against 96,
-// 4096 x 4096 29 against 33, 8192 x 8192 the same; 20 x 50000 11.5 against
-// 7.3, so few long rows take the look-back variants).  One sequence: the
-// table's variant 9 fits about 8.4 million elements; beyond, the same entry's
-// `tile` is the shape of variant 8.
+// A scan's variant.  The table is keyed by the total size alone; rules add
+// what it cannot see.  Rows: one block per row (variant 9) wherever a row fits
+// a block's shared memory and either there is a row for every second SM or a
+// row is short (4097 x 4099 38 us against 298, 8192 x 256 9 against 96, 4096 x
+// 4096 29 against 33, 8192 x 8192 the same; 20 x 50000 11.5 against 7.3).
+// Where the table names variant 9 (2^18 to 2^24 elements) and it does not
+// apply:
+//   few long rows   look-back tiles, of 16 KiB below 2^20 elements (variant 4;
+//                   20 x 50000 float32 7.4 us, 5 8.1), of 48 KiB below 2^22
+//                   (variant 5; 70 x 20000 8.3 us, 8 18.6 to 20.4; 4 x 300000
+//                   8.1, 8 10.2 to 11.8), else variant 8
+//   one sequence    variant 8: more than the 8.4 million elements that fit the
+//                   SMs' shared memory
+// Variant 8 in the shape that is best up to 2^24 (8.5 million 18.8 us, the
+// others 19.8).
 int dispatch_scan(const ScanLaunch &sc, const Context &ctx, cudaStream_t s)
 {
     return run_with_fallback(SKEL_SK_SCAN, ctx, [&](const Choice &c) { return launch_scan(sc, c, s); }, scan_def,
@@ -543,8 +550,10 @@ int dispatch_scan(const ScanLaunch &sc, const Context &ctx, cudaStream_t s)
                                  const bool fits = scan_wave_fits(sc), rows = sc.seg > 0 && sc.seg < sc.n;
                                  if (rows && fits && (sc.seg <= 8192 || sc.n / sc.seg >= device_info().sms / 2))
                                      c = Choice{9, 256, 4, 0};
-                                 else if (c.variant == 9 && (rows || !fits))   // variant 4 below 2^20 elements
-                                     c = sc.n < (1 << 20) ? Choice{4, 256, 4, 0} : Choice{8, 256, 4, c.tile};
+                                 else if (c.variant == 9 && (rows || !fits))
+                                     c = rows && sc.n < (1 << 20)   ? Choice{4, 256, 4, 0}
+                                         : rows && sc.n < (1 << 22) ? Choice{5, 256, 4, 3}
+                                                                    : Choice{8, 256, 4, 1};
                              });
 }
 
