@@ -162,7 +162,8 @@ class ComposedLossFn(torch.autograd.Function):
     of the separate calls and only t is saved.
 
     `step(name, thunk)`, when given, runs each call (the benchmark times
-    them one by one); the calls and their order are the same either way."""
+    them one by one): fwd_fused and bwd_fused, or the calls above; which of
+    the two does not depend on it."""
 
     @staticmethod
     def forward(ctx, x, weights, boundary: str, step=None):
