@@ -592,7 +592,7 @@ def launch_floor(sk, torch, stream, count: int = 200) -> float:
 
 def l2_random_rate(sk, torch, stream, m: int = 1 << 20, reads: int = 1 << 28):
     """Random 4-byte reads per second from an L2-resident table of m floats
-    (the gather's table size): the gather's measured ceiling."""
+    (the gather's table size) that miss L1: the gather's measured ceiling."""
     dev = torch.device("cuda")
     table = torch.from_numpy(syn.uniform_f32(syn.SEED_X + 8, m)).to(dev)
     sink = torch.zeros(1, device=dev)
@@ -1008,10 +1008,11 @@ def main():
             g_rate = N / (g_ms * 1e-3)
             l2["gather_frac"] = round(g_rate / rate, 3)
             if dom[0] == "maparray_gather":
-                # the gather's table reads are random L2 sectors: its roofline is
-                # the measured random-read rate, in the gather's own units (8
-                # algorithmic bytes per read: the index read and the output write)
-                roofline = {"bound": "l2", "kernel": dom[0], "achieved": round(dom_gbs, 1),
+                # the gather's table reads miss L1, one sector each, and an SM takes
+                # one such sector per clock: the roofline is the measured random-read
+                # rate, in the gather's own units (8 algorithmic bytes per read: the
+                # index read and the output write)
+                roofline = {"bound": "l1_miss", "kernel": dom[0], "achieved": round(dom_gbs, 1),
                             "peak": round(8 * rate / 1e9, 1), "unit": "GB/s", "frac": round(g_rate / rate, 3),
                             "peak_kind": "measured (skel_probe_l2_random), 8 algorithmic bytes per random read",
                             "hbm_peak": hbm, "hbm_frac": round(dom_gbs / hbm, 3), "traffic": committed_traffic(dom[0])}

@@ -6,9 +6,13 @@
 //                      (the latency bound of the small MapReduce).
 //   probe_l2_random    random 4-byte reads from a table that stays in L2
 //                      (MapArray gather's access pattern without its index
-//                      and output streams): the L2's random-sector rate, the
-//                      roofline of the gather.  Indices come from a per-thread
-//                      generator in registers, so no HBM stream competes.
+//                      and output streams): the roofline of the gather.
+//                      Indices come from a per-thread generator in registers,
+//                      so no HBM stream competes.  A table that misses L1 gives
+//                      3.1e11 reads/s from 2^17 to 2^24 floats, which is one
+//                      sector per SM and clock; 2 SMs reach the same rate each
+//                      as 152 do (0.97), so the bound is the SM's path to L2,
+//                      not L2.  Tables in L1 give 8.8e11 (2^15 floats) and more.
 #include "common.cuh"
 
 namespace skel {
