@@ -460,7 +460,14 @@ int skel_mapoverlap_bwd(skel_fn fn, int radius, const float *weights, int nweigh
  * replace the built-in defaults for their key; a call whose key has no entry
  * uses the entry of the nearest lower tuned bucket of the same (skeleton, fn,
  * dtype, radius, residency), else the nearest higher one, else the built-in
- * default.  path NULL clears the table (built-in defaults only). */
+ * default.  path NULL clears the table (built-in defaults only).
+ * Two kinds of calls also go by what the key does not show, whatever the
+ * table says (a forced variant still applies): row-wise scans run one block
+ * per row (variant 9) where a row fits a block's shared memory and rows are
+ * short or many, and batched calls for which the table names variant 7 run
+ * variant 0 with at most 512 instances and fewer than 2^23 elements.  Where
+ * the table names scan variant 9 and it does not fit, a look-back variant
+ * runs. */
 int skel_load_dispatch_table(const char *path);
 
 /* Adds or replaces one table entry (same fields as a table line). */

@@ -27,8 +27,8 @@
 // What bounds it (8192 x 8192): the forward takes 127 us, the backward 174
 // (180 and 235 with cp.async), against 79 us each for their HBM traffic
 // (which ncu shows at 1.0 of the algorithmic bytes): instruction issue, active
-// 71 and 61 % of the time, with 16 warps per SM whose barriers keep them in the
-// same phase (52 and 63 instructions per 32 points: two MUFUs and about 15
+// 71 and 64 % of the time, with 16 warps per SM whose barriers keep them in the
+// same phase (52 and 64 instructions per 32 points: two MUFUs and about 15
 // others of tanhf, 9 FMAs per stencil, 5 to 6 per scan).  The forward
 // therefore splits its barrier into an arrival and a wait, with the stencil's
 // inner columns and the next row's tanh between them (136 us with one whole
